@@ -599,36 +599,60 @@ constexpr int kBoundsPerGroup = kN0Max + kN0Max * kN1Max;
 // Centre index of a lane's segment [st, st + g) inside [.., end) (end = its last state + 1).
 __device__ __forceinline__ int segment_centre(int st, int g, int end) { return min(st + g / 2, min(st + g, end) - 1); }
 
-// The warp's bounding sphere of one segment: lanes with `has` hold their seed's segment centre
-// (x, y, z); the sphere is centred on the midpoint of the first and the last such lane's centres
-// (opposite corners of the lattice block, so about the middle of the group's tracks), its radius
-// is the largest distance to any lane's centre plus `reach` (a state within g/2 recording intervals
-// of a centre is at most (g/2) h_rec from it along the track).  Any centre gives a valid sphere;
-// the radius is measured from the centre as rounded, and rounded up so that it never shrinks; in
-// double the rounding of the centre to float is added.  Returns radius < 0 when no lane has the
-// segment.
+// A group's spread about a segment's centre states: the midpoint of two of its lanes' centres, the
+// square m2 of the largest distance from it to any lane's centre, and rs about 1 / sqrt(m2).
+template <typename T>
+struct WarpSpread {
+    T cx, cy, cz;
+    float m2, rs;
+};
+
+// Lanes with `has` hold their seed's segment centre (x, y, z), l0 and l1 are the first and the last
+// such lane (opposite corners of the lattice block, so the midpoint lies about the middle of the
+// group's tracks).
+template <typename T>
+__device__ __forceinline__ WarpSpread<T> warp_spread(bool has, int l0, int l1, T x, T y, T z)
+{
+    WarpSpread<T> w;
+    w.cx = T(0.5) * (__shfl_sync(0xffffffffu, x, l0) + __shfl_sync(0xffffffffu, x, l1));
+    w.cy = T(0.5) * (__shfl_sync(0xffffffffu, y, l0) + __shfl_sync(0xffffffffu, y, l1));
+    w.cz = T(0.5) * (__shfl_sync(0xffffffffu, z, l0) + __shfl_sync(0xffffffffu, z, l1));
+    // d^2 >= 0 as a float (rounded up from double): its bit pattern orders like its value, so one
+    // integer warp reduction finds the max; then one root by the hardware reciprocal square root
+    // (a few ulp, inside the 1e-6 relative margin of the radius).  The radius is a float either way,
+    // so the double path needs no double root or reductions (this part's FP64 rate is small).
+    float d2;
+    if constexpr (sizeof(T) == 4)
+        d2 = has ? (x - w.cx) * (x - w.cx) + (y - w.cy) * (y - w.cy) + (z - w.cz) * (z - w.cz) : 0.f;
+    else
+        d2 = has ? __double2float_ru((x - w.cx) * (x - w.cx) + (y - w.cy) * (y - w.cy) + (z - w.cz) * (z - w.cz)) : 0.f;
+    w.m2 = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(d2)));
+    w.rs = rsqrtf(fmaxf(w.m2, 1e-30f));
+    return w;
+}
+
+// The bounding sphere of a segment: centred on the spread's midpoint, its radius the largest distance
+// plus `reach` (a state within g/2 recording intervals of a centre is at most (g/2) h_rec from it along
+// the track).  Any centre gives a valid sphere; the radius is measured from the centre as rounded, and
+// rounded up so that it never shrinks; in double the rounding of the centre to float is added.
+template <typename T>
+__device__ __forceinline__ float4 spread_sphere(const WarpSpread<T> &w, T reach)
+{
+    float rad;
+    if constexpr (sizeof(T) == 4)
+        rad = __fmul_rn(__fmaf_rn(w.m2, w.rs, reach), 1.000001f);
+    else
+        rad = (float)(((T)(w.m2 * w.rs) + reach + T(2e-7)) * T(1.000001));
+    return make_float4((float)w.cx, (float)w.cy, (float)w.cz, rad);
+}
+
+// The warp's bounding sphere of one segment; radius < 0 when no lane has the segment.
 template <typename T>
 __device__ __forceinline__ float4 warp_sphere(bool has, T x, T y, T z, T reach)
 {
     const uint32_t hm = __ballot_sync(0xffffffffu, has);
     if (hm == 0u) return make_float4(0.f, 0.f, 0.f, -1.f);
-    const int l0 = __ffs(hm) - 1, l1 = 31 - __clz(hm);
-    const T cx = T(0.5) * (__shfl_sync(0xffffffffu, x, l0) + __shfl_sync(0xffffffffu, x, l1));
-    const T cy = T(0.5) * (__shfl_sync(0xffffffffu, y, l0) + __shfl_sync(0xffffffffu, y, l1));
-    const T cz = T(0.5) * (__shfl_sync(0xffffffffu, z, l0) + __shfl_sync(0xffffffffu, z, l1));
-    // d^2 >= 0 as a float (rounded up from double): its bit pattern orders like its value, so one
-    // integer warp reduction finds the max; then one root by the hardware reciprocal square root
-    // (a few ulp, inside the 1e-6 relative margin below).  The radius is a float either way, so the
-    // double path needs no double root or reductions (this part's FP64 rate is small).
-    float d2;
-    if constexpr (sizeof(T) == 4)
-        d2 = has ? (x - cx) * (x - cx) + (y - cy) * (y - cy) + (z - cz) * (z - cz) : 0.f;
-    else
-        d2 = has ? __double2float_ru((x - cx) * (x - cx) + (y - cy) * (y - cy) + (z - cz) * (z - cz)) : 0.f;
-    const float m2 = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(d2)));
-    const T d = (T)(m2 * rsqrtf(fmaxf(m2, 1e-30f)));
-    const T extra = sizeof(T) == 8 ? T(2e-7) : T(0);
-    return make_float4((float)cx, (float)cy, (float)cz, (float)((d + reach + extra) * T(1.000001)));
+    return spread_sphere<T>(warp_spread<T>(has, __ffs(hm) - 1, 31 - __clz(hm), x, y, z), reach);
 }
 
 // ------------------------------------------------------------------------------------------------

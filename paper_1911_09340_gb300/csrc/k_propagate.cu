@@ -277,7 +277,142 @@ __device__ __forceinline__ void advance_interval(const F &f, const PropArgs &a, 
     }
 }
 
+// Whether a track in a uniform axial field provably stays inside the target region for all its n_rec
+// states.  One recording interval is X' = X + N P, P' = M P (axial_interval), so the states lie on
+// X_k = C + G M^k P_0 with G = N / (M - 1) and C = X_0 - G P_0: within |C| + |G P_0| |M|^k of the axis, and
+// z moves by dz per interval.  Tested in float whatever the working precision: the margins (0.1 mm, 4 nm
+// per state and 2e-6 of the coordinates; |M|^k from |M|^2 - 1 plus its rounding) are far above the
+// float rounding here and the rounding of the recorded states.  A track near the boundary, a straight one
+// (M = 1) or one that is not finite keeps the per-state test.
+__device__ __forceinline__ bool stays_inside(float x, float y, float z, float px, float py,
+                                             const AxialStep<float> &k, int n_rec, float zmin, float zmax,
+                                             float rmax2)
+{
+    const float den = k.am1 * k.am1 + k.b * k.b;
+    const float n = (float)n_rec;
+    const float grow = 0.5f * (fmaxf(2.f * k.am1 + den, 0.f) + 4e-7f) * n;
+    if (!(den > 1e-10f && grow < 0.05f)) return false;
+    const float inv = 1.f / den;
+    const float gr = (k.c * k.am1 + k.d * k.b) * inv, gi = (k.c * k.b - k.d * k.am1) * inv;
+    const float cx = x - (gr * px - gi * py), cy = y - (gr * py + gi * px);
+    const float rr = sqrtf((gr * gr + gi * gi) * (px * px + py * py));
+    const float z1 = z + (n - 1.f) * k.dz;
+    float rout = sqrtf(cx * cx + cy * cy) + rr * (1.f + 1.1f * grow);
+    const float margin = 1e-4f + 4e-9f * n + 2e-6f * (rout + fabsf(z) + fabsf(z1));
+    rout += margin;
+    return rout * rout < rmax2 && fminf(z, z1) > zmin + margin && fmaxf(z, z1) < zmax - margin;
+}
+
+// The recording of a warp whose 32 tracks all stay inside (stays_inside): no per-state region test, no
+// per-lane activity, every lane in every sphere, so nothing in the loop depends on the lane but the
+// arithmetic.  Off: the byte offset of a value inside its plane, 32 bits when the planes are small enough
+// (one addition per state then serves the six stores).  With one-state segments two states are recorded
+// before their two spheres are formed, so that the two chains of shuffles and reductions overlap (a
+// few seeds leave one warp per scheduler, which has nothing else to issue).  Bound by the stores at
+// 2^18 seeds and by the issue of one warp per scheduler at a few thousand.  FP32 with spheres, before
+// (the general loop of propagate_kernel) and after: 2^18 seeds x 70 states 101 -> 82 us (5.2 TB/s of
+// stores), 2^14 x 2229 386 -> 160 us, 256 x 70 25 -> 15 us; FP64 2^15 x 139 427 -> 359 us.
+template <typename T, class F, int STRIDE, typename Off>
+__device__ __forceinline__ void record_inside(const F &f, const PropArgs &a, const AxialStep<T> &ks, T y[6],
+                                              bool valid, int64_t s, int lane, float4 *tab, T R0, T R1)
+{
+    const int n_rec = a.n_rec, G0 = a.G0, G1 = a.G1;
+    const int64_t plane = (int64_t)n_rec * a.S;
+    T *const p0 = (T *)a.points, *const p1 = p0 + plane, *const p2 = p1 + plane, *const p3 = p2 + plane,
+             *const p4 = p3 + plane, *const p5 = p4 + plane;
+    Off off = (Off)s * (Off)sizeof(T);
+    const Off row = (Off)a.S * (Off)sizeof(T);
+    float lo[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    typename F::Cell cell;
+    auto store = [&]() {
+        if (valid) {
+            *(T *)((char *)p0 + off) = y[0];
+            *(T *)((char *)p1 + off) = y[1];
+            *(T *)((char *)p2 + off) = y[2];
+            *(T *)((char *)p3 + off) = y[3];
+            *(T *)((char *)p4 + off) = y[4];
+            *(T *)((char *)p5 + off) = y[5];
+        }
+    };
+    auto next = [&]() {
+        advance_interval<T, F, STRIDE>(f, a, ks, T(0), T(0), T(0), y, lo, cell);
+        off += row;
+        store();
+    };
+    store();
+    int r = 0;
+    if (!tab) {
+#pragma unroll 4
+        for (r = 1; r < n_rec; ++r) next();
+        return;
+    }
+    // entries that no segment fills
+    const int n0 = (n_rec + G0 - 1) / G0;
+    for (int i = lane; i < kBoundsPerGroup; i += 32) {
+        const int j = i < kN0Max ? i : (i - kN0Max) / kN1Max, m = i < kN0Max ? 0 : (i - kN0Max) % kN1Max;
+        if (j >= n0 || m * G1 >= min(G0, n_rec - j * G0)) tab[i] = make_float4(0.f, 0.f, 0.f, -1.f);
+    }
+    int j = 0, c0 = segment_centre(0, G0, min(G0, n_rec));   // current super-segment and its centre
+    auto super = [&](const WarpSpread<T> &w) {
+        if (lane == 0) tab[j] = spread_sphere<T>(w, R0);
+        ++j;
+        c0 = j < n0 ? segment_centre(j * G0, G0, min(j * G0 + G0, n_rec)) : 0x7fffffff;
+    };
+    float4 *t1 = tab + kN0Max;   // next level-1 entry
+    int m = 0;
+    if (G1 == 1) {
+        auto emit = [&](const WarpSpread<T> &w, int k) {
+            if (lane == 0) *t1 = spread_sphere<T>(w, R1);
+            ++t1;
+            if (++m == G0) {
+                m = 0;
+                t1 += kN1Max - G0;
+            }
+            if (k == c0) super(w);
+        };
+        emit(warp_spread<T>(true, 0, 31, y[0], y[1], y[2]), 0);
+        for (r = 1; r + 1 < n_rec; r += 2) {
+            next();
+            const T x1 = y[0], y1 = y[1], z1 = y[2];
+            next();
+            const WarpSpread<T> wa = warp_spread<T>(true, 0, 31, x1, y1, z1);
+            const WarpSpread<T> wb = warp_spread<T>(true, 0, 31, y[0], y[1], y[2]);
+            emit(wa, r);
+            emit(wb, r + 1);
+        }
+        if (r < n_rec) {
+            next();
+            emit(warp_spread<T>(true, 0, 31, y[0], y[1], y[2]), r);
+        }
+        return;
+    }
+    int st1 = 0, se1 = min(G0, n_rec), c1 = segment_centre(0, G1, se1), j1 = 0;
+    for (;;) {
+        // to the next centre (of a level-1 or a super-segment), or the end
+        const int to = min(min(c0, c1), n_rec - 1);
+#pragma unroll 4
+        for (; r < to; ++r) next();
+        if (r != c0 && r != c1) return;
+        const WarpSpread<T> w = warp_spread<T>(true, 0, 31, y[0], y[1], y[2]);
+        if (r == c1) {
+            if (lane == 0) t1[j1 * kN1Max + m] = spread_sphere<T>(w, R1);
+            ++m;
+            st1 += G1;
+            if (st1 >= se1) {
+                m = 0;
+                st1 = ++j1 * G0;
+                se1 = min(st1 + G0, n_rec);
+            }
+            c1 = st1 < n_rec ? segment_centre(st1, G1, se1) : 0x7fffffff;
+        }
+        if (r == c0) super(w);
+    }
+}
+
 // BATCH: one launch for a batch of events; block b belongs to the event that batch_find gives.
+// Lanes past the last seed repeat it without storing: with idle lanes instead, the shuffles of every
+// sphere found the last warp of a seed count that is no multiple of 32 diverged, and that one warp
+// made the launch 4 times as long (10,000 seeds x 140 states: 191 us against 46 us for 9,984).
 template <typename T, class F, int STRIDE, bool BATCH>
 __global__ void __launch_bounds__(128) propagate_kernel(F f, PropArgs a, BatchLaunch L)
 {
@@ -289,31 +424,28 @@ __global__ void __launch_bounds__(128) propagate_kernel(F f, PropArgs a, BatchLa
         a = L.ev[e].prop;
         bx = lb;
     }
-    const int64_t s = bx * blockDim.x + threadIdx.x;
-    const int lane = threadIdx.x & 31;
-    const bool valid = s < a.S;
-    const bool wb = a.bounds != nullptr;   // whole warps then stay in the loop (warp reductions)
-    if (!valid && !wb) return;
-    // a warp with no seed at all (past the end) has no bounds entry: it leaves as a whole
-    if ((s & ~(int64_t)31) >= a.S) return;
     const int64_t S = a.S;
+    int64_t s = bx * blockDim.x + threadIdx.x;
+    const int lane = threadIdx.x & 31;
+    const bool valid = s < S;
+    // a warp with no seed at all (past the end) has no bounds entry: it leaves as a whole
+    if ((s & ~(int64_t)31) >= S) return;
+    s = valid ? s : S - 1;
+    const bool wb = a.bounds != nullptr;   // whole warps then stay in the loop (warp reductions)
     const T *__restrict__ seeds = (const T *)a.seeds;
     T *__restrict__ pts = (T *)a.points;
     const int64_t plane = (int64_t)a.n_rec * S;
     const int n_rec = a.n_rec;
 
-    T y[6] = {T(0), T(0), T(0), T(0), T(0), T(0)};
-    int q = 0;
-    if (valid) {
+    T y[6];
 #pragma unroll
-        for (int c = 0; c < 6; ++c) y[c] = seeds[c * S + s];
-        q = a.charge[s];
-    }
+    for (int c = 0; c < 6; ++c) y[c] = seeds[c * S + s];
+    const int q = a.charge[s];
     constexpr bool kFF = sizeof(T) == 4 && F::kAxial;   // FP32 axial: no double arithmetic at all
     T c = T(0), ip = T(0);
     double ipd = 1.0;
     if constexpr (!kFF) {
-        const double pd = valid ? sqrt((double)y[3] * y[3] + (double)y[4] * y[4] + (double)y[5] * y[5]) : 1.0;
+        const double pd = sqrt((double)y[3] * y[3] + (double)y[4] * y[4] + (double)y[5] * y[5]);
         ipd = 1.0 / pd;
         c = (T)(kKappa * q * ipd);
         ip = (T)ipd;
@@ -325,8 +457,7 @@ __global__ void __launch_bounds__(128) propagate_kernel(F f, PropArgs a, BatchLa
     // uniform axial field: the interval's map is fixed per seed
     AxialStep<T> ks{};
     if constexpr (kFF) {
-        ks = axial_interval_ff(y[3], y[4], y[5], valid ? q : 0, f.bz, a.h_ff,
-                               STRIDE > 0 ? STRIDE : a.stride);
+        ks = axial_interval_ff(y[3], y[4], y[5], q, f.bz, a.h_ff, STRIDE > 0 ? STRIDE : a.stride);
     } else if constexpr (F::kAxial) {
         const double w = kKappa * q * (double)f.bz * ipd;
         const double t = a.h * w, t2 = t * t, hp = a.h * ipd;
@@ -339,13 +470,26 @@ __global__ void __launch_bounds__(128) propagate_kernel(F f, PropArgs a, BatchLa
         ks.d = (T)m[3];
         ks.dz = (T)m[4];
     }
+    float4 *tab = wb ? (float4 *)a.bounds + (s >> 5) * kBoundsPerGroup : nullptr;
+    if constexpr (F::kAxial) {
+        const AxialStep<float> kf{(float)ks.am1, (float)ks.b, (float)ks.c, (float)ks.d, (float)ks.dz};
+        const bool in = stays_inside((float)y[0], (float)y[1], (float)y[2], (float)y[3], (float)y[4], kf, n_rec,
+                                     a.lim_f[0], a.lim_f[1], a.lim_f[2]);
+        if (__all_sync(0xffffffffu, in)) {
+            if (valid) a.n_valid[s] = n_rec;
+            if (plane * (int64_t)sizeof(T) < ((int64_t)1 << 32))
+                record_inside<T, F, STRIDE, uint32_t>(f, a, ks, y, valid, s, lane, tab, R0, R1);
+            else
+                record_inside<T, F, STRIDE, size_t>(f, a, ks, y, valid, s, lane, tab, R0, R1);
+            return;
+        }
+    }
     float lo[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};   // FP32: low words of the compensated state
     typename F::Cell cell;                          // tabulated field: the cell of the last lookup
 
     // Bounding spheres of the segments whose centre is the state just recorded (see device.cuh);
     // lanes that stopped earlier contribute their last recorded state if the segment holds it.
     // The next centres are tracked incrementally.
-    float4 *tab = wb ? (float4 *)a.bounds + (s >> 5) * kBoundsPerGroup : nullptr;
     int last_k = 0;
     const int G0 = a.G0, G1 = a.G1;
     int j1 = 0, m1 = 0, st1 = 0, se1 = min(G0, n_rec);   // current level-1 segment
@@ -362,13 +506,15 @@ __global__ void __launch_bounds__(128) propagate_kernel(F f, PropArgs a, BatchLa
         for (int cc = 0; cc < 6; ++cc) pts[cc * plane + s] = y[cc];
     }
     int n = 1;
-    bool active = valid && !outside_region<T>(y[0], y[1], y[2], zmin, zmax, rmax2);
+    bool active = !outside_region<T>(y[0], y[1], y[2], zmin, zmax, rmax2);
     for (int r = 0; r < n_rec; ++r) {
         if (r > 0 && active) {
             advance_interval<T, F, STRIDE>(f, a, ks, c, ip, h, y, lo, cell);
             const int64_t o = (int64_t)r * S + s;
+            if (valid) {
 #pragma unroll
-            for (int cc = 0; cc < 6; ++cc) pts[cc * plane + o] = y[cc];
+                for (int cc = 0; cc < 6; ++cc) pts[cc * plane + o] = y[cc];
+            }
             n = r + 1;
             last_k = r;
             if (outside_region<T>(y[0], y[1], y[2], zmin, zmax, rmax2)) active = false;
@@ -376,14 +522,14 @@ __global__ void __launch_bounds__(128) propagate_kernel(F f, PropArgs a, BatchLa
         if (wb) {
             if (G1 == 1) {
                 // every recorded state is a level-1 segment of its own: (j1, m1) = (r / G0, r % G0)
-                const float4 sp = warp_sphere<T>(valid && last_k >= r, y[0], y[1], y[2], R1);
+                const float4 sp = warp_sphere<T>(last_k >= r, y[0], y[1], y[2], R1);
                 if (lane == 0) tab[kN0Max + j1 * kN1Max + m1] = sp;
                 if (++m1 == G0) {
                     m1 = 0;
                     ++j1;
                 }
             } else if (r == c1) {
-                const float4 sp = warp_sphere<T>(valid && last_k >= st1, y[0], y[1], y[2], R1);
+                const float4 sp = warp_sphere<T>(last_k >= st1, y[0], y[1], y[2], R1);
                 if (lane == 0) tab[kN0Max + j1 * kN1Max + m1] = sp;
                 ++m1;
                 st1 += G1;
@@ -396,7 +542,7 @@ __global__ void __launch_bounds__(128) propagate_kernel(F f, PropArgs a, BatchLa
                 c1 = st1 < n_rec ? segment_centre(st1, G1, se1) : 0x7fffffff;
             }
             if (r == c0) {
-                const float4 sp = warp_sphere<T>(valid && last_k >= sb0, y[0], y[1], y[2], R0);
+                const float4 sp = warp_sphere<T>(last_k >= sb0, y[0], y[1], y[2], R0);
                 if (lane == 0) tab[j0] = sp;
                 ++j0;
                 sb0 += G0;
