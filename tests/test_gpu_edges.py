@@ -42,3 +42,23 @@ def test_recording_inside_the_region_equals_the_tested_one(ctx, dtype, stride, n
     for a, b in zip(free, edge):
         assert torch.equal(a, b)
     assert bool((free[1] == bp.n_rec).all())
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.float64])
+@pytest.mark.parametrize("S", [64, 65, 127, 2048 + 63, 2 * 2048 + 1, 40 * 2048 + 5])
+@pytest.mark.parametrize("k", [2, 32, 33, 64])
+def test_top_k_lists(ctx, dtype, S, k):
+    """The warps' sorted lists of 64 against the oracle's selection: a last chunk shorter than k, list
+    halves, signed zeros (equal, so by index), infinities and NaN, descending input (every key enters)."""
+    rng = np.random.default_rng(S + k)
+    special = rng.choice(np.array([0.0, -0.0, np.inf, np.nan, 1.5, -2.0, 3.0]), size=S)
+    for v in (special, np.arange(S, 0, -1, dtype=np.float64)):
+        v = v.astype(np.float32 if dtype == torch.float32 else np.float64)
+        rss = torch.as_tensor(v, device="cuda")
+        idx = torch.full((k,), -7, dtype=torch.int64, device="cuda")
+        val = torch.zeros(k, dtype=dtype, device="cuda")
+        B.comet_scan_select(ctx, rss, k, idx, val)
+        order = np.lexsort((np.arange(S), np.where(np.isnan(v), 0.0, v), np.isnan(v)))[:k]
+        assert np.array_equal(idx.cpu().numpy(), order)
+        assert np.array_equal(val.cpu().numpy(), v[order], equal_nan=True)
+        assert np.array_equal(np.signbit(val.cpu().numpy()), np.signbit(v[order]))
