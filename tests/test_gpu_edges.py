@@ -62,3 +62,26 @@ def test_top_k_lists(ctx, dtype, S, k):
         assert np.array_equal(idx.cpu().numpy(), order)
         assert np.array_equal(val.cpu().numpy(), v[order], equal_nan=True)
         assert np.array_equal(np.signbit(val.cpu().numpy()), np.signbit(v[order]))
+
+
+@pytest.mark.parametrize("M", [1, 127, 128, 129, 700])
+@pytest.mark.parametrize("half_width", [(0.03125, 0.5, 2.0, 3.0), (0.015625, 1.6, 1.5, 5.0), (0.0, 0.0, 0.0, 0.0)])
+def test_reference_walk_over_tiles(ctx, M, half_width):
+    """References from more candidates than one tile, with unused slots and with z0 and pz on a lattice
+    (differences that equal the width exactly) and phi across the +-pi seam, against the oracle."""
+    rng = np.random.default_rng(M)
+    n = 900
+    z, phi = rng.integers(-8, 9, n) / 64.0, rng.uniform(-np.pi, np.pi, n)
+    pz, pt = np.round(rng.uniform(10, 20, n)), rng.uniform(95, 105, n)
+    seeds = np.stack([0 * z, 0 * z, z, pt * np.cos(phi), pt * np.sin(phi), pz], axis=1)
+    idx = rng.integers(-2, n + 2, size=M)
+    idx[0] = 5
+    K = 32
+    refs = torch.zeros((K, 4), dtype=torch.float64, device="cuda")
+    nref = torch.zeros(1, dtype=torch.int32, device="cuda")
+    dev = torch.as_tensor(np.ascontiguousarray(seeds.T), device="cuda")
+    B.comet_scan_refine_refs(ctx, dev, torch.as_tensor(idx, device="cuda"), half_width, K, refs, nref)
+    got = refs[: int(nref)].cpu().numpy()
+    want = O.refine_refs(seeds, idx, half_width, K)
+    assert got.shape == want.shape
+    assert np.allclose(got, want, rtol=1e-14, atol=1e-14)
