@@ -275,6 +275,32 @@ __device__ __forceinline__ void axial_increment(const AxialStep<T> &k, const T y
     inc[5] = T(0);
 }
 
+// Whether a track in a uniform axial field provably stays inside the target region for all its n_rec
+// states.  One recording interval is X' = X + N P, P' = M P (axial_interval), so the states lie on
+// X_k = C + G M^k P_0 with G = N / (M - 1) and C = X_0 - G P_0: within |C| + |G P_0| |M|^k of the axis, and
+// z moves by dz per interval.  Tested in float whatever the working precision: the margins (0.1 mm,
+// per_state for each state's rounding and 2e-6 of the coordinates; |M|^k from |M|^2 - 1 plus its
+// rounding) are far above the float rounding here and the rounding of the recorded states.  A track near
+// the boundary, a straight one (M = 1) or one that is not finite keeps the per-state test.
+__device__ __forceinline__ bool stays_inside(float x, float y, float z, float px, float py,
+                                             const AxialStep<float> &k, int n_rec, float zmin, float zmax,
+                                             float rmax2, float per_state)
+{
+    const float den = k.am1 * k.am1 + k.b * k.b;
+    const float n = (float)n_rec;
+    const float grow = 0.5f * (fmaxf(2.f * k.am1 + den, 0.f) + 4e-7f) * n;
+    if (!(den > 1e-10f && grow < 0.05f)) return false;
+    const float inv = 1.f / den;
+    const float gr = (k.c * k.am1 + k.d * k.b) * inv, gi = (k.c * k.b - k.d * k.am1) * inv;
+    const float cx = x - (gr * px - gi * py), cy = y - (gr * py + gi * px);
+    const float rr = sqrtf((gr * gr + gi * gi) * (px * px + py * py));
+    const float z1 = z + (n - 1.f) * k.dz;
+    float rout = sqrtf(cx * cx + cy * cy) + rr * (1.f + 1.1f * grow);
+    const float margin = 1e-4f + per_state * n + 2e-6f * (rout + fabsf(z) + fabsf(z1));
+    rout += margin;
+    return rout * rout < rmax2 && fminf(z, z1) > zmin + margin && fmaxf(z, z1) < zmax - margin;
+}
+
 // The four stages of one classic RK4 step of length h from state y, the field from look(x, y, z,
 // bx, by, bz): inc = h/6 (k1 + 2 k2 + 2 k3 + k4).  c = KAPPA q / P0, ip = 1 / P0.
 template <typename T, class Look>

@@ -3,18 +3,22 @@
 // The seed is parameterised by theta = (z0, phi, pz, pT) with the vertex (vx, vy) fixed, as in the
 // lattice.  With P = px + i py and X = x + i y, one RK4 step of length h in B = (0, 0, Bz) is the
 // linear map P' = m P, X' = X + n P, z' = z + dz, whose coefficients depend on P0 = |p| and h only
-// (device.cuh); the k-th recorded state is therefore P_k = M^k P_0, X_k = X_0 + N (M^k - 1)/(M - 1)
-// P_0 with (M, N) the map of one recording interval.  Carrying every quantity as a value plus its
-// four partial derivatives in theta (forward mode) gives the derivatives of the recorded states in
-// closed form.
+// (device.cuh), and so do those of any product of steps: after a path of length L, X = X_0 + N P_0 and
+// z = z_0 + L pz / |p|.  The derivatives of the recorded states in theta therefore need the maps'
+// derivatives in one variable, |p|: the path is carried as X and P, each with its derivative in ln(1/|p|)
+// (forward mode), and the chain rule in (z0, phi, pz, pT) is applied once, at its end.  This part's FP64
+// unit holds its scheduler for 64 cycles per warp instruction, whatever the active lanes, so the
+// kernel's time is its longest lane's count of FP64 instructions: carrying four derivatives through
+// every step and through the maps' powers took 225 us for 16 seeds x 100 wires.  A whole call, 16 seeds x
+// 134 wires x 138 states 438 -> 95 us, 64 x 134 x 2229 584 -> 232 us, 1000 x 134 x 138 1856 -> 663 us.
 //
 // The DCA of a wire is the distance at the point of closest approach (PCA) found as in the scan: the
 // closest recorded state (searched in FP32, settled in FP64 among its neighbours), then the local
 // virtual-plane Newton refinement of Algorithm 2, each refinement step being one RK4 step of the
 // axial map.  At the PCA the distance
 // is stationary along the track, so dD/dtheta = nhat . dx/dtheta at the fixed arc length of the PCA
-// (envelope theorem): the refinement steps are replayed in forward mode with their lengths held
-// fixed.  nhat is the unit vector from the wire to the PCA.
+// (envelope theorem): the refinement steps enter the product of maps with their lengths held fixed.
+// nhat is the unit vector from the wire to the PCA.
 //
 // Smoothed residual (Eq. 1 with a differentiable cap): e = min_j |D - r_j| over the wire's unmasked
 // hits, w = sigmoid((lambda - e) / tau), term = w e^2 + (1 - w) lambda^2.  Gauss-Newton treats w as
@@ -28,228 +32,215 @@ namespace comet {
 
 namespace {
 
-// value + 4 partial derivatives
-struct D4 {
-    double v, d[4];
+// A complex number and its derivative D = -P0 d/dP0.
+struct Cd {
+    double re, im, dre, dim;
 };
 
-__device__ __forceinline__ D4 dc(double v) { return D4{v, {0.0, 0.0, 0.0, 0.0}}; }
-__device__ __forceinline__ D4 operator+(const D4 &a, const D4 &b)
+// a + m b
+__device__ __forceinline__ Cd mul_add(const Cd &a, const Cd &m, const Cd &b)
 {
-    return D4{a.v + b.v, {a.d[0] + b.d[0], a.d[1] + b.d[1], a.d[2] + b.d[2], a.d[3] + b.d[3]}};
-}
-__device__ __forceinline__ D4 operator-(const D4 &a, const D4 &b)
-{
-    return D4{a.v - b.v, {a.d[0] - b.d[0], a.d[1] - b.d[1], a.d[2] - b.d[2], a.d[3] - b.d[3]}};
-}
-__device__ __forceinline__ D4 operator-(const D4 &a) { return D4{-a.v, {-a.d[0], -a.d[1], -a.d[2], -a.d[3]}}; }
-__device__ __forceinline__ D4 operator*(const D4 &a, const D4 &b)
-{
-    D4 r;
-    r.v = a.v * b.v;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) r.d[j] = a.d[j] * b.v + a.v * b.d[j];
-    return r;
-}
-__device__ __forceinline__ D4 operator*(double s, const D4 &a)
-{
-    return D4{s * a.v, {s * a.d[0], s * a.d[1], s * a.d[2], s * a.d[3]}};
-}
-__device__ __forceinline__ D4 operator/(const D4 &a, const D4 &b)
-{
-    D4 r;
-    const double ib = 1.0 / b.v;
-    r.v = a.v * ib;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) r.d[j] = (a.d[j] - r.v * b.d[j]) * ib;
-    return r;
-}
-__device__ __forceinline__ D4 dsqrt(const D4 &a)
-{
-    D4 r;
-    r.v = sqrt(a.v);
-    const double k = r.v > 0.0 ? 0.5 / r.v : 0.0;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) r.d[j] = a.d[j] * k;
-    return r;
+    return Cd{a.re + (m.re * b.re - m.im * b.im), a.im + (m.re * b.im + m.im * b.re),
+              a.dre + ((m.dre * b.re - m.dim * b.im) + (m.re * b.dre - m.im * b.dim)),
+              a.dim + ((m.dre * b.im + m.dim * b.re) + (m.re * b.dim + m.im * b.dre))};
 }
 
-// complex number of D4 parts
-struct C4 {
-    D4 re, im;
-};
-__device__ __forceinline__ C4 operator+(const C4 &a, const C4 &b) { return C4{a.re + b.re, a.im + b.im}; }
-__device__ __forceinline__ C4 operator*(const C4 &a, const C4 &b)
-{
-    return C4{a.re * b.re - a.im * b.im, a.re * b.im + a.im * b.re};
-}
-__device__ __forceinline__ C4 cdiv(const C4 &a, const C4 &b)
-{
-    const D4 den = b.re * b.re + b.im * b.im;
-    return C4{(a.re * b.re + a.im * b.im) / den, (a.im * b.re - a.re * b.im) / den};
-}
-
-// One RK4 step of length h in the axial field: P' = m P, X' = X + n P, z' = z + dz, with m = 1 + A.
-struct StepMap {
-    C4 A, n;   // A = m - 1 = am1 - i b, n = c - i d
-    D4 dz;
+// The map of a path: P' = (1 + A) P, X' = X + N P.
+struct PathMap {
+    Cd A, N;
 };
 
-__device__ __forceinline__ StepMap step_map(const D4 &P0, const D4 &pz, double h, double kqb)
+// One RK4 step of length h: A = m - 1 = -t^2 (1/2 - t^2/24) - i t (1 - t^2/6), N = hp (1 - t^2/6) -
+// i hp t (1/2 - t^2/24), with t = h w and hp = h / P0 (w and 1 / P0 both have D = themselves).
+__device__ __forceinline__ PathMap step_map(double ip, double w, double h)
 {
-    const D4 ip = dc(1.0) / P0;
-    const D4 t = (h * kqb) * ip;
-    const D4 t2 = t * t;
-    const D4 hp = h * ip;
-    const D4 g = dc(1.0) - (1.0 / 6.0) * t2;
-    StepMap s;
-    s.A.re = t2 * (dc(-0.5) + (1.0 / 24.0) * t2);
-    s.A.im = -(t * g);
-    s.n.re = hp * g;
-    s.n.im = -(hp * t * (dc(0.5) - (1.0 / 24.0) * t2));
-    s.dz = hp * pz;
-    return s;
+    const double t = h * w, t2 = t * t, hp = h * ip;
+    const double u = 1.0 - t2 * (1.0 / 6.0), v = 0.5 - t2 * (1.0 / 24.0), q = 1.0 - 0.5 * t2;
+    const double tu = t * u;
+    return PathMap{Cd{-(t2 * v), -tu, -(t2 * u), -(t * q)}, Cd{hp * u, -(hp * (t * v)), hp * q, -(hp * tu)}};
 }
 
-// (1 + A)^k - 1 by binary powering on A ((1 + a)(1 + b) - 1 = a + b + a b: nothing cancels)
-__device__ __forceinline__ C4 pow_minus_one(const C4 &A, int k)
+__device__ __forceinline__ void cmul(double ar, double ai, double br, double bi, double &r, double &i)
 {
-    C4 R{dc(0.0), dc(0.0)}, Bp = A;
-    bool first = true;
-    for (int e = k; e > 0; e >>= 1) {
-        if (e & 1) {
-            if (first) {
-                R = Bp;
-                first = false;
-            } else {
-                R = R + Bp + R * Bp;
+    r = ar * br - ai * bi;
+    i = ar * bi + ai * br;
+}
+__device__ __forceinline__ void crecip(double re, double im, double &r, double &i)
+{
+    const double inv = 1.0 / (re * re + im * im);
+    r = re * inv;
+    i = -im * inv;
+}
+
+// Passes of one map s: A_k = (1 + A)^k - 1 by binary powering on values ((1 + a)(1 + b) - 1 = a + b + a b:
+// nothing cancels), N_k = N S with S = A_k / A, and from them D A_k = k (1 + A_k) q with q = DA / (1 + A)
+// and D S = (D A_k - S DA) / A: the derivatives cost the same whatever k.
+struct Powers {
+    PathMap s;
+    double ir, ii, qr, qi;   // 1 / A and q
+    bool turns;
+    __device__ __forceinline__ explicit Powers(const PathMap &m) : s(m)
+    {
+        turns = s.A.re != 0.0 || s.A.im != 0.0;
+        crecip(s.A.re, s.A.im, ir, ii);
+        double r, i;
+        crecip(1.0 + s.A.re, s.A.im, r, i);
+        cmul(s.A.dre, s.A.dim, r, i, qr, qi);
+    }
+    __device__ __forceinline__ PathMap operator()(int k) const   // k >= 0
+    {
+        double Rr = 0.0, Ri = 0.0, Br = s.A.re, Bi = s.A.im;
+        for (int e = k; e > 0; e >>= 1) {
+            double r, i;
+            if (e & 1) {
+                cmul(Rr, Ri, Br, Bi, r, i);
+                Rr = (Rr + Br) + r;
+                Ri = (Ri + Bi) + i;
+            }
+            if (e > 1) {
+                cmul(Br, Bi, Br, Bi, r, i);
+                Br = 2.0 * Br + r;
+                Bi = 2.0 * Bi + i;
             }
         }
-        if (e > 1) Bp = Bp + Bp + Bp * Bp;
+        PathMap m;
+        Cd S{(double)k, 0.0, 0.0, 0.0};
+        m.A = Cd{Rr, Ri, 0.0, 0.0};
+        if (turns) {
+            cmul(1.0 + Rr, Ri, (double)k * qr, (double)k * qi, m.A.dre, m.A.dim);
+            cmul(Rr, Ri, ir, ii, S.re, S.im);
+            double r, i;
+            cmul(S.re, S.im, s.A.dre, s.A.dim, r, i);
+            cmul(m.A.dre - r, m.A.dim - i, ir, ii, S.dre, S.dim);
+        }
+        m.N = mul_add(Cd{0.0, 0.0, 0.0, 0.0}, s.N, S);
+        return m;
     }
-    return R;
-}
-
-// k steps of a map (same coefficients): A_k = (1 + A)^k - 1, n_k = n (A_k / A), dz_k = k dz
-__device__ __forceinline__ StepMap power_map(const StepMap &s, int k)
-{
-    StepMap r;
-    r.A = pow_minus_one(s.A, k);
-    const bool turns = s.A.re.v != 0.0 || s.A.im.v != 0.0;
-    const C4 S = turns ? cdiv(r.A, s.A) : C4{dc((double)k), dc(0.0)};
-    r.n = s.n * S;
-    r.dz = (double)k * s.dz;
-    return r;
-}
-
-struct State4 {
-    C4 X, P;
-    D4 z;
 };
 
-__device__ __forceinline__ State4 apply(const StepMap &s, const State4 &y)
-{
-    State4 o;
-    o.X = y.X + s.n * y.P;
-    o.P = y.P + s.A * y.P;
-    o.z = y.z + s.dz;
-    return o;
-}
-
-// value-only version of a step: (x, y, z, px, py) += the map
-struct Step1 {
-    double am1, b, c, d, dz;
+// A path from the seed per unit of transverse momentum: X = X_0 + pT x, P = pT p, both functions of P0 at
+// a fixed phi.
+struct Path {
+    Cd x, p;
 };
-__device__ __forceinline__ Step1 step1(double P0, double pz, double h, double kqb)
+__device__ __forceinline__ void apply(const PathMap &s, Path &y)
 {
-    const double t = h * kqb / P0, t2 = t * t, hp = h / P0, g = 1.0 - t2 / 6.0;
-    return Step1{t2 * (-0.5 + t2 / 24.0), t * g, hp * g, hp * t * (0.5 - t2 / 24.0), hp * pz};
+    y.x = mul_add(y.x, s.N, y.p);
+    y.p = mul_add(y.p, s.A, y.p);
 }
-__device__ __forceinline__ void apply1(const Step1 &s, double y[5])
+// values only
+__device__ __forceinline__ void apply_values(const PathMap &s, Path &y)
 {
-    const double px = y[3], py = y[4];
-    y[0] += s.c * px + s.d * py;
-    y[1] += s.c * py - s.d * px;
-    y[2] += s.dz;
-    y[3] += s.am1 * px + s.b * py;
-    y[4] += s.am1 * py - s.b * px;
+    const double pr = y.p.re, pi = y.p.im;
+    y.x.re += s.N.re * pr - s.N.im * pi;
+    y.x.im += s.N.re * pi + s.N.im * pr;
+    y.p.re += s.A.re * pr - s.A.im * pi;
+    y.p.im += s.A.re * pi + s.A.im * pr;
 }
 
-constexpr int kMaxSteps = 64;   // refinement steps replayed in forward mode (max_iter is capped)
+constexpr int kMaxSteps = 64;    // refinement steps at most (max_iter is capped)
+constexpr int kWalkTile = 256;   // recorded states staged at a time
 
-__global__ void __launch_bounds__(32) jacobian_kernel(JacArgs a)
+// One warp: one seed and 32 of its wires, or with few wires 32 / G seeds and G >= W lanes for each (G a
+// power of two), so that no more than half the lanes idle.  Lanes past the last wire or seed repeat it
+// without writing.
+__global__ void __launch_bounds__(32) jacobian_kernel(JacArgs a, int G)
 {
-    const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (tid >= a.S * a.W) return;
-    const int64_t s = tid / a.W;
-    const int i = (int)(tid % a.W);
-    double *out = a.work + tid * 11;   // flag, term, dterm, w, rho, J[0..3], nhat_x, nhat_y
-    const int hb = a.offs[i], he = a.offs[i + 1];
-    bool any = false;
-    for (int j = hb; j < he; ++j) any = any || !a.mask[j];
+    __shared__ float4 walk_s[kWalkTile];
+    const int chunks = (a.W + G - 1) / G;
+    const int g = threadIdx.x / G, lane = threadIdx.x & (G - 1);   // lane of the group
+    const int64_t sg = (int64_t)(blockIdx.x / chunks) * (32 / G) + g;
+    const int i = (int)(blockIdx.x % chunks) * G + lane;
+    const bool has = i < a.W && sg < a.S;
+    const int64_t s = sg < a.S ? sg : a.S - 1;
+    const int iw = i < a.W ? i : a.W - 1;
+    const int tile = kWalkTile / 32 * G;
+    float4 *walk = walk_s + g * tile;
 
-    // seed and its derivatives: theta = (z0, phi, pz, pT)
+    // seed: theta = (z0, phi, pz, pT)
     const double *th = a.theta + s * 4;
-    const double cphi = cos(th[1]), sphi = sin(th[1]);
-    State4 y0;
-    y0.X = C4{dc(a.vx), dc(a.vy)};
-    y0.P.re = D4{th[3] * cphi, {0.0, -th[3] * sphi, 0.0, cphi}};
-    y0.P.im = D4{th[3] * sphi, {0.0, th[3] * cphi, 0.0, sphi}};
-    y0.z = D4{th[0], {1.0, 0.0, 0.0, 0.0}};
-    const D4 pz = D4{th[2], {0.0, 0.0, 1.0, 0.0}};
-    const D4 pt = D4{th[3], {0.0, 0.0, 0.0, 1.0}};
-    const D4 P0 = dsqrt(pt * pt + pz * pz);
-    const double kqb = kKappa * a.charge * a.bz;
-    const StepMap one = step_map(P0, pz, a.h, kqb);
-    const StepMap itv = power_map(one, a.stride);
+    const double z0 = th[0], pz = th[2], pt = th[3];
+    double sphi, cphi;
+    sincos(th[1], &sphi, &cphi);
+    const double P0 = sqrt(pt * pt + pz * pz), ip = 1.0 / P0;
+    const double w = kKappa * a.charge * a.bz * ip;
+    const PathMap one = step_map(ip, w, a.h);
+    const Powers itv(a.stride == 1 ? one : Powers(one)(a.stride));
+    const double tz = pz * ip, tt = pt * ip;
+    const double dz = (double)a.stride * (a.h * tz);
 
     // wire
-    const double *w = (const double *)a.wires;
-    const double ax = w[0 * a.ldw + i], ay = w[1 * a.ldw + i], az = w[2 * a.ldw + i];
-    const double ux = w[3 * a.ldw + i], uy = w[4 * a.ldw + i], uz = w[5 * a.ldw + i];
+    const double *wr = (const double *)a.wires + iw;
+    const double ax = wr[0 * a.ldw], ay = wr[1 * a.ldw], az = wr[2 * a.ldw];
+    const double ux = wr[3 * a.ldw], uy = wr[4 * a.ldw], uz = wr[5 * a.ldw];
 
     // closest recorded state, recording as the scan does: state 0, then each interval, stopping
     // after the first state outside the target region.  The walk runs in FP32 (FP64 instructions
-    // are scarce on this part); the argmin is then settled in FP64 among the FP32 choice and its
-    // two neighbours.
-    const double pzv = pz.v;
-    const float am1f = (float)itv.A.re.v, bbf = (float)-itv.A.im.v, ccf = (float)itv.n.re.v,
-                ddf = (float)-itv.n.im.v, dzf = (float)itv.dz.v;
-    float f[5] = {(float)y0.X.re.v, (float)y0.X.im.v, (float)y0.z.v, (float)y0.P.re.v, (float)y0.P.im.v};
+    // are scarce on this part), the seed's states once into shared memory and then each lane's wire
+    // against them; the argmin is settled in FP64 among the FP32 choice and its two neighbours.
+    const float am1f = (float)itv.s.A.re, bbf = (float)-itv.s.A.im, ccf = (float)itv.s.N.re,
+                ddf = (float)-itv.s.N.im, dzf = (float)dz;
+    float f[5] = {(float)a.vx, (float)a.vy, (float)z0, (float)(pt * cphi), (float)(pt * sphi)};
     const float axf = (float)ax, ayf = (float)ay, azf = (float)az, uxf = (float)ux, uyf = (float)uy,
                 uzf = (float)uz;
     const float zminf = (float)a.zmin, zmaxf = (float)a.zmax, rmax2f = (float)a.rmax2;
     float bestf = INFINITY;
     int kbest = 0, nvalid = a.n_rec;
-    for (int k = 0; k < a.n_rec; ++k) {
-        if (k > 0) {
-            const float px = f[3], py = f[4];
-            f[0] += ccf * px + ddf * py;
-            f[1] += ccf * py - ddf * px;
-            f[2] += dzf;
-            f[3] += am1f * px + bbf * py;
-            f[4] += am1f * py - bbf * px;
+    auto step = [&]() {
+        const float px = f[3], py = f[4];
+        f[0] += ccf * px + ddf * py;
+        f[1] += ccf * py - ddf * px;
+        f[2] += dzf;
+        f[3] += am1f * px + bbf * py;
+        f[4] += am1f * py - bbf * px;
+    };
+    // a track that provably stays inside the region needs no test per state (0.1 um of rounding per
+    // plain float state)
+    const bool inside = stays_inside(f[0], f[1], f[2], f[3], f[4], AxialStep<float>{am1f, bbf, ccf, ddf, dzf},
+                                     a.n_rec, zminf, zmaxf, rmax2f, 1e-7f);
+    for (int kt = 0; __any_sync(0xffffffffu, kt < nvalid); kt += tile) {
+        const int ke = min(kt + tile, nvalid);
+        int k = kt;
+        if (inside) {
+#pragma unroll 4
+            for (; k < ke; ++k) {
+                if (k > 0) step();
+                if (lane == (k & (G - 1))) walk[k - kt] = make_float4(f[0], f[1], f[2], 0.f);
+            }
+        } else {
+            for (; k < ke; ++k) {
+                if (k > 0) step();
+                if (lane == (k & (G - 1))) walk[k - kt] = make_float4(f[0], f[1], f[2], 0.f);
+                if (f[2] < zminf || f[2] > zmaxf || f[0] * f[0] + f[1] * f[1] > rmax2f) {
+                    nvalid = ++k;
+                    break;
+                }
+            }
         }
-        const float d2 = line_dist2<float>(f[0], f[1], f[2], axf, ayf, azf, uxf, uyf, uzf);
-        if (d2 < bestf) {
-            bestf = d2;
-            kbest = k;
+        __syncwarp();
+#pragma unroll 4
+        for (int j = 0; j < k - kt; ++j) {
+            const float4 p = walk[j];
+            const float d2 = line_dist2<float>(p.x, p.y, p.z, axf, ayf, azf, uxf, uyf, uzf);
+            if (d2 < bestf) {
+                bestf = d2;
+                kbest = kt + j;
+            }
         }
-        if (f[2] < zminf || f[2] > zmaxf || f[0] * f[0] + f[1] * f[1] > rmax2f) {
-            nvalid = k + 1;
-            break;
-        }
+        __syncwarp();
     }
-    // FP64 (forward mode): states kbest - 1 .. kbest + 1, the lowest distance, ties to the lower index
+    // FP64: states kbest - 1 .. kbest + 1, the lowest distance, ties to the lower index
     const int k0 = kbest > 0 ? kbest - 1 : 0;
-    const State4 base = k0 > 0 ? apply(power_map(itv, k0), y0) : y0;
+    Path y{Cd{0.0, 0.0, 0.0, 0.0}, Cd{cphi, sphi, 0.0, 0.0}};
+    apply(itv(k0), y);
     {
         double best = INFINITY;
         int kb = kbest;
-        State4 cur = base;
+        Path c = y;
         for (int k = k0; k <= kbest + 1 && k < nvalid; ++k) {
-            if (k > k0) cur = apply(itv, cur);
-            const double d2 = line_dist2<double>(cur.X.re.v, cur.X.im.v, cur.z.v, ax, ay, az, ux, uy, uz);
+            if (k > k0) apply_values(itv.s, c);
+            const double d2 = line_dist2<double>(a.vx + pt * c.x.re, a.vy + pt * c.x.im, z0 + (double)k * dz, ax, ay,
+                                                 az, ux, uy, uz);
             if (d2 < best) {
                 best = d2;
                 kb = k;
@@ -257,24 +248,22 @@ __global__ void __launch_bounds__(32) jacobian_kernel(JacArgs a)
         }
         kbest = kb;
     }
-    State4 yk = base;
-    for (int k = k0; k < kbest; ++k) yk = apply(itv, yk);
+    for (int k = k0; k < kbest; ++k) apply(itv.s, y);
 
-    // local virtual-plane refinement (values), remembering the step lengths
-    double y[6] = {yk.X.re.v, yk.X.im.v, yk.z.v, yk.P.re.v, yk.P.im.v, pzv};
-    double ds_list[kMaxSteps];
-    int n_ds = 0, conv = 0;
+    // local virtual-plane refinement from there, on the position relative to the wire's point
+    const double vx = a.vx - ax, vy = a.vy - ay, vz = (z0 - az) + (double)kbest * dz;
+    int conv = 0;
     double sigma = 0.0;
     const int max_iter = a.max_iter < kMaxSteps ? a.max_iter : kMaxSteps;
     for (int it = 0;; ++it) {
-        const double rp = 1.0 / sqrt(y[3] * y[3] + y[4] * y[4] + y[5] * y[5]);
-        const double tx = y[3] * rp, ty = y[4] * rp, tz = y[5] * rp;
+        // t = p / P0: |p| stays P0 in a magnetic field (refine_dca)
+        const double tx = tt * y.p.re, ty = tt * y.p.im;
         const double tu = tx * ux + ty * uy + tz * uz;
         const double nx = tx - tu * ux, ny = ty - tu * uy, nz = tz - tu * uz;
         const double nn2 = nx * nx + ny * ny + nz * nz;
         if (nn2 < 1e-18) break;
-        const double rn = 1.0 / sqrt(nn2);
-        const double dist = ((y[0] - ax) * nx + (y[1] - ay) * ny + (y[2] - az) * nz) * rn;
+        const double rn = rsqrt(nn2);
+        const double dist = ((vx + pt * y.x.re) * nx + (vy + pt * y.x.im) * ny + (vz + sigma * tz) * nz) * rn;
         if (fabs(dist) < a.tol) {
             conv = 1;
             break;
@@ -285,39 +274,43 @@ __global__ void __launch_bounds__(32) jacobian_kernel(JacArgs a)
         target = target < -a.h_rec ? -a.h_rec : target;
         const double ds = target - sigma;
         if (ds == 0.0) break;
-        const Step1 st = step1(P0.v, pzv, ds, kqb);
-        double y5[5] = {y[0], y[1], y[2], y[3], y[4]};
-        apply1(st, y5);
-        for (int c = 0; c < 5; ++c) y[c] = y5[c];
-        ds_list[n_ds++] = ds;
+        apply(step_map(ip, w, ds), y);
         sigma = target;
     }
-    // replay the steps in forward mode at their fixed lengths
-    for (int q = 0; q < n_ds; ++q) yk = apply(step_map(P0, pz, ds_list[q], kqb), yk);
 
-    // D and dD/dtheta = nhat . dx/dtheta
-    const double rx = yk.X.re.v - ax, ry = yk.X.im.v - ay, rz = yk.z.v - az;
+    // D and dD/dtheta = nhat . dx/dtheta at the path's fixed length
+    const double rx = vx + pt * y.x.re, ry = vy + pt * y.x.im, rz = vz + sigma * tz;
     const double al = rx * ux + ry * uy + rz * uz;
     const double ex = rx - al * ux, ey = ry - al * uy, ez = rz - al * uz;
     const double D = sqrt(ex * ex + ey * ey + ez * ez);
     const double inv = D > 0.0 ? 1.0 / D : 0.0;
+    const double hx = ex * inv, hy = ey * inv, hz = ez * inv;
+    // X = X_0 + pT x: dX/dphi = i pT x, dX/dpT = x + pT dx/dP0 dP0/dpT, dX/dpz = pT dx/dP0 dP0/dpz;
+    // z = z_0 + L pz / P0, so dz/dpz = (L / P0) (1 - tz^2), dz/dpT = -(L / P0) tz tt
+    const double hq = -tt * (hx * y.x.dre + hy * y.x.dim);   // nhat . pT dx/dP0
+    const double lz = (((double)kbest * a.stride) * a.h + sigma) * ip * hz;
     double J[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j)
-        J[j] = (ex * yk.X.re.d[j] + ey * yk.X.im.d[j] + ez * yk.z.d[j]) * inv;
+    J[0] = hz;
+    J[1] = pt * (hy * y.x.re - hx * y.x.im);
+    J[2] = hq * tz + lz * (1.0 - tz * tz);
+    J[3] = hq * tt + (hx * y.x.re + hy * y.x.im) - lz * tz * tt;
 
     // smoothed residual of the wire
+    if (!has) return;
+    const int hb = a.offs[i], he = a.offs[i + 1];
+    bool any = false;
+    double e = INFINITY, r_best = 0.0;
+    for (int j = hb; j < he; ++j) {
+        if (a.mask[j]) continue;
+        any = true;
+        const double ej = fabs(D - a.drift[j]);
+        if (ej < e) {
+            e = ej;
+            r_best = a.drift[j];
+        }
+    }
     double term = 0.0, dterm = 0.0, wgt = 0.0, rho = 0.0;
     if (any) {
-        double e = INFINITY, r_best = 0.0;
-        for (int j = hb; j < he; ++j) {
-            if (a.mask[j]) continue;
-            const double ej = fabs(D - a.drift[j]);
-            if (ej < e) {
-                e = ej;
-                r_best = a.drift[j];
-            }
-        }
         const double lam = a.lambda;
         wgt = 1.0 / (1.0 + exp(-(lam - e) / a.tau));
         term = wgt * e * e + (1.0 - wgt) * lam * lam;
@@ -326,6 +319,8 @@ __global__ void __launch_bounds__(32) jacobian_kernel(JacArgs a)
         dterm = sgn * (2.0 * wgt * e + dw * (e * e - lam * lam));
         rho = D - r_best;
     }
+    const int64_t tid = s * a.W + i;
+    double *out = a.work + tid * 11;   // flag, term, dterm, w, rho, J[0..3], nhat_x, nhat_y
     out[0] = any ? 1.0 : 0.0;
     out[1] = term;
     out[2] = dterm;
@@ -338,49 +333,68 @@ __global__ void __launch_bounds__(32) jacobian_kernel(JacArgs a)
     }
 #pragma unroll
     for (int j = 0; j < 4; ++j) out[5 + j] = J[j];
-    out[9] = ex * inv;    // dD/dx0 and dD/dy0: the recorded X_k depend on (x0, y0) additively
-    out[10] = ey * inv;
+    out[9] = hx;    // dD/dx0 and dD/dy0: the recorded X_k depend on (x0, y0) additively
+    out[10] = hy;
     if (!conv && any && a.n_unconv) atomicAdd(a.n_unconv, 1);
 }
 
-// per seed, ascending wire order: smoothed RSS, its gradient, J^T W J and J^T W rho
-__global__ void jacobian_reduce_kernel(JacArgs a)
+// Per seed, ascending wire order: smoothed RSS, its gradient, J^T W J and J^T W rho.  One warp per seed: the
+// terms of 32 wires at a time go to shared memory, then lane q adds product q of the 27 sums wire by
+// wire (the order, and the one rounding per product, of a single thread doing them all, which waited
+// on memory for every wire: 210 us for 16 seeds x 100 wires).
+__global__ void __launch_bounds__(32) jacobian_reduce_kernel(JacArgs a)
 {
-    const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= a.S) return;
-    double srss = 0.0, g[4] = {0, 0, 0, 0}, jtj[16], jtr[4] = {0, 0, 0, 0}, gxy[2] = {0, 0};
-    for (int q = 0; q < 16; ++q) jtj[q] = 0.0;
-    for (int i = 0; i < a.W; ++i) {
-        const int64_t t = s * a.W + i;
-        const double *o = a.work + t * 11;
-        if (o[0] == 0.0) continue;
-        const double *J = o + 5;
-        srss += o[1];
-        gxy[0] += o[2] * o[9];
-        gxy[1] += o[2] * o[10];
-        for (int j = 0; j < 4; ++j) {
-            g[j] += o[2] * J[j];
-            jtr[j] += o[3] * o[4] * J[j];
-            for (int k = 0; k < 4; ++k) jtj[j * 4 + k] += o[3] * J[j] * J[k];
+    // factors of a wire's products: f[0] = 1, [1] = dterm, [2] = w rho, [3..6] = w J, g[0] = term,
+    // [1..4] = J, [5..6] = nhat
+    __shared__ double sf[32][7], sg[32][7];
+    __shared__ int any[32];
+    const int64_t s = blockIdx.x;
+    const int q = threadIdx.x;
+    // sum q: 0 smoothed RSS, 1-4 gradient, 5-8 J^T W rho, 9-24 J^T W J, 25-26 gradient in (x0, y0)
+    const int fi = q == 0 ? 0 : q < 5 ? 1 : q < 9 ? 2 : q < 25 ? 3 + (q - 9) / 4 : 1;
+    const int gi = q == 0 ? 0 : q < 5 ? q : q < 9 ? q - 4 : q < 25 ? 1 + (q - 9) % 4 : q < 27 ? q - 20 : 0;
+    double acc = 0.0;
+    for (int i0 = 0; i0 < a.W; i0 += 32) {
+        const int n = min(32, a.W - i0);
+        if (q < n) {
+            const double *o = a.work + (s * a.W + i0 + q) * 11;
+            any[q] = o[0] != 0.0;
+            sf[q][0] = 1.0;
+            sf[q][1] = o[2];
+            sf[q][2] = o[3] * o[4];
+            sg[q][0] = o[1];
+            sg[q][5] = o[9];
+            sg[q][6] = o[10];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                sf[q][3 + j] = o[3] * o[5 + j];
+                sg[q][1 + j] = o[5 + j];
+            }
         }
+        __syncwarp();
+        for (int t = 0; t < n; ++t)
+            if (any[t]) acc = fma(sf[t][fi], sg[t][gi], acc);
+        __syncwarp();
     }
-    a.srss_out[s] = srss;
-    for (int j = 0; j < 4; ++j) {
-        a.grad_out[s * 4 + j] = g[j];
-        a.jtr_out[s * 4 + j] = jtr[j];
-    }
-    for (int q = 0; q < 16; ++q) a.jtj_out[s * 16 + q] = jtj[q];
+    if (q == 0) a.srss_out[s] = acc;
+    else if (q < 5) a.grad_out[s * 4 + q - 1] = acc;
+    else if (q < 9) a.jtr_out[s * 4 + q - 5] = acc;
+    else if (q < 25) a.jtj_out[s * 16 + q - 9] = acc;
     if (a.grad6_out) {
         // (x0, y0, z0, px, py, pz): phi = atan2(py, px) and pT = hypot(px, py), by the chain rule
+        double g[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) g[j] = __shfl_sync(0xffffffffu, acc, 1 + j);
         const double phi = a.theta[s * 4 + 1], pt = a.theta[s * 4 + 3];
         const double cp = cos(phi), sp = sin(phi);
         double *o = a.grad6_out + s * 6;
-        o[0] = gxy[0];
-        o[1] = gxy[1];
-        o[2] = g[0];
-        o[3] = -g[1] * sp / pt + g[3] * cp;
-        o[4] = g[1] * cp / pt + g[3] * sp;
-        o[5] = g[2];
+        if (q == 25 || q == 26) o[q - 25] = acc;
+        if (q == 0) {
+            o[2] = g[0];
+            o[3] = -g[1] * sp / pt + g[3] * cp;
+            o[4] = g[1] * cp / pt + g[3] * sp;
+            o[5] = g[2];
+        }
     }
 }
 
@@ -460,14 +474,16 @@ __global__ void lm_step_kernel(LmArgs a)
 
 cudaError_t launch_jacobian(const JacArgs &a, cudaStream_t st)
 {
-    const int64_t n = a.S * a.W;
-    if (n > 0) {
-        // small blocks: a few thousand threads of long FP64 chains, spread over as many SMs as possible
-        jacobian_kernel<<<(unsigned)((n + 31) / 32), 32, 0, st>>>(a);
+    if (a.W > 0) {
+        // one warp per block: a few dozen warps of long FP64 chains, spread over as many SMs as possible
+        int G = 32;
+        while (G > 1 && G / 2 >= a.W) G /= 2;
+        const int64_t blocks = (a.S + 32 / G - 1) / (32 / G) * ((a.W + G - 1) / G);
+        jacobian_kernel<<<(unsigned)blocks, 32, 0, st>>>(a, G);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
-    jacobian_reduce_kernel<<<(unsigned)((a.S + 63) / 64), 64, 0, st>>>(a);
+    jacobian_reduce_kernel<<<(unsigned)a.S, 32, 0, st>>>(a);
     return cudaGetLastError();
 }
 

@@ -277,32 +277,6 @@ __device__ __forceinline__ void advance_interval(const F &f, const PropArgs &a, 
     }
 }
 
-// Whether a track in a uniform axial field provably stays inside the target region for all its n_rec
-// states.  One recording interval is X' = X + N P, P' = M P (axial_interval), so the states lie on
-// X_k = C + G M^k P_0 with G = N / (M - 1) and C = X_0 - G P_0: within |C| + |G P_0| |M|^k of the axis, and
-// z moves by dz per interval.  Tested in float whatever the working precision: the margins (0.1 mm, 4 nm
-// per state and 2e-6 of the coordinates; |M|^k from |M|^2 - 1 plus its rounding) are far above the
-// float rounding here and the rounding of the recorded states.  A track near the boundary, a straight one
-// (M = 1) or one that is not finite keeps the per-state test.
-__device__ __forceinline__ bool stays_inside(float x, float y, float z, float px, float py,
-                                             const AxialStep<float> &k, int n_rec, float zmin, float zmax,
-                                             float rmax2)
-{
-    const float den = k.am1 * k.am1 + k.b * k.b;
-    const float n = (float)n_rec;
-    const float grow = 0.5f * (fmaxf(2.f * k.am1 + den, 0.f) + 4e-7f) * n;
-    if (!(den > 1e-10f && grow < 0.05f)) return false;
-    const float inv = 1.f / den;
-    const float gr = (k.c * k.am1 + k.d * k.b) * inv, gi = (k.c * k.b - k.d * k.am1) * inv;
-    const float cx = x - (gr * px - gi * py), cy = y - (gr * py + gi * px);
-    const float rr = sqrtf((gr * gr + gi * gi) * (px * px + py * py));
-    const float z1 = z + (n - 1.f) * k.dz;
-    float rout = sqrtf(cx * cx + cy * cy) + rr * (1.f + 1.1f * grow);
-    const float margin = 1e-4f + 4e-9f * n + 2e-6f * (rout + fabsf(z) + fabsf(z1));
-    rout += margin;
-    return rout * rout < rmax2 && fminf(z, z1) > zmin + margin && fmaxf(z, z1) < zmax - margin;
-}
-
 // The recording of a warp whose 32 tracks all stay inside (stays_inside): no per-state region test, no
 // per-lane activity, every lane in every sphere, so nothing in the loop depends on the lane but the
 // arithmetic.  Off: the byte offset of a value inside its plane, 32 bits when the planes are small enough
@@ -474,7 +448,7 @@ __global__ void __launch_bounds__(128) propagate_kernel(F f, PropArgs a, BatchLa
     if constexpr (F::kAxial) {
         const AxialStep<float> kf{(float)ks.am1, (float)ks.b, (float)ks.c, (float)ks.d, (float)ks.dz};
         const bool in = stays_inside((float)y[0], (float)y[1], (float)y[2], (float)y[3], (float)y[4], kf, n_rec,
-                                     a.lim_f[0], a.lim_f[1], a.lim_f[2]);
+                                     a.lim_f[0], a.lim_f[1], a.lim_f[2], 4e-9f);
         if (__all_sync(0xffffffffu, in)) {
             if (valid) a.n_valid[s] = n_rec;
             if (plane * (int64_t)sizeof(T) < ((int64_t)1 << 32))

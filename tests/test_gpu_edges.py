@@ -85,3 +85,40 @@ def test_reference_walk_over_tiles(ctx, M, half_width):
     want = O.refine_refs(seeds, idx, half_width, K)
     assert got.shape == want.shape
     assert np.allclose(got, want, rtol=1e-14, atol=1e-14)
+
+
+@pytest.mark.parametrize("n_seeds,n_wires,stride", [(1, 1, 16), (5, 2, 1), (7, 3, 16), (3, 16, 4), (2, 33, 16), (65, 5, 32)])
+def test_jacobian_lane_groups(ctx, n_seeds, n_wires, stride):
+    """Few wires share a warp between seeds (2^n lanes each), more than 32 take several warps: the DCAs are
+    the oracle's to 1e-9 m where the refinement converges, and the sums are those of the per-wire
+    values in ascending wire order."""
+    ev = synth.single_event_fp64()
+    spec = ev.partitions[0]
+    rng = np.random.default_rng(n_seeds)
+    theta = np.array(spec.centre) + rng.uniform(-0.2, 0.2, (n_seeds, 4)) * np.array(spec.half_width)
+    near = np.nonzero([np.any(ev.hit_turn[a:b] == 0) for a, b in zip(ev.hit_offsets[:-1], ev.hit_offsets[1:])])[0]
+    wires = ev.wires[:, near[:n_wires]]
+    W = wires.shape[1]
+    assert W == n_wires
+    drift = rng.uniform(0.0, 8e-3, W)
+    lam, tau = 1e-2, 1e-3
+    p = B.ScanParams(n_steps=ev.n_steps[0], stride=stride, lam=lam)
+    f64 = dict(dtype=torch.float64, device="cuda")
+    t = lambda x, d=torch.float64: torch.as_tensor(np.ascontiguousarray(x), dtype=d, device="cuda")
+    work, D, J = torch.empty(n_seeds * W * 11, **f64), torch.empty((n_seeds, W), **f64), torch.empty((n_seeds, W, 4), **f64)
+    srss, grad, jtj, jtr = (torch.empty(s, **f64) for s in (n_seeds, (n_seeds, 4), (n_seeds, 16), (n_seeds, 4)))
+    B.comet_scan_jacobian(ctx, B.DeviceField.from_synth(UNIFORM), p, t(theta), *spec.vxy, spec.charge, t(wires),
+                          t(np.arange(W + 1), torch.int32), t(drift), t(np.zeros(W), torch.uint8), tau, work, srss,
+                          grad, jtj, jtr, dca_out=D, jac_out=J)
+    seeds = np.stack([np.full(n_seeds, spec.vxy[0]), np.full(n_seeds, spec.vxy[1]), theta[:, 0],
+                      theta[:, 3] * np.cos(theta[:, 1]), theta[:, 3] * np.sin(theta[:, 1]), theta[:, 2]], axis=1)
+    ref = O.scan(UNIFORM, O.Params(n_steps=ev.n_steps[0], stride=stride, lam=lam), seeds, spec.charge,
+                 O.wires_aos(wires), np.arange(W + 1, dtype=np.int32), drift, np.zeros(W, np.uint8), want_dca=True)
+    D, J = D.cpu().numpy(), J.cpu().numpy()
+    assert np.abs(D - ref["dca"]).max() <= 1e-9
+    rho = D - drift
+    e = np.abs(rho)
+    w = 1.0 / (1.0 + np.exp(-(lam - e) / tau))
+    assert np.allclose(srss.cpu(), (w * e * e + (1 - w) * lam * lam).sum(1), rtol=1e-12)
+    assert np.allclose(jtr.cpu(), ((w * rho)[..., None] * J).sum(1), rtol=1e-10, atol=1e-12)
+    assert np.allclose(jtj.cpu().numpy().reshape(-1, 4, 4), np.einsum("sw,swi,swj->sij", w, J, J), rtol=1e-10, atol=1e-12)
