@@ -17,6 +17,7 @@
  *                         one turn partition of many events in single launches
  *   comet_scan_classify   classify the selected seed's hits; mask them for the next   (Sec. 2.1, 3.1)
  *                         turn partition
+ *   comet_scan_partition  the five of one turn partition in one call
  *
  * Conventions shared by every call
  *   - Units: metres, MeV/c, tesla.  Equations of motion in arc length s, with P0 = |p| of the seed
@@ -433,6 +434,22 @@ comet_status comet_scan_batch(comet_ctx *ctx, comet_dtype dtype, const comet_fie
  *   other host threads) race on the array: serialise them. */
 comet_status comet_scan_select_noalloc(comet_dtype dtype, const void *rss, int64_t S, int32_t k,
                                        int64_t *idx_out, void *rss_out, comet_stream stream);
+
+/* ---- one turn partition ---------------------------------------------------------------------------
+ * comet_scan_partition: comet_scan_lattice, comet_scan_propagate, comet_scan_dca, comet_scan_select and
+ *   comet_scan_classify in this order on `stream`, with the arguments of the same names (arrays, checks
+ *   and results as theirs).  k = 1: the seed of lowest RSS is selected in the DCA launch (best_idx_out,
+ *   best_rss_out of comet_scan_dca); k > 1: comet_scan_select writes idx_out [k] and rss_out [k].
+ *   The classified seed is idx_out[0].  The first step that fails ends the call with its status; the
+ *   steps before it are enqueued. */
+comet_status comet_scan_partition(comet_ctx *ctx, comet_dtype dtype, const comet_field *field,
+                                  const comet_scan_params *params, const comet_lattice *lat, int32_t k,
+                                  void *seeds, int8_t *charge, int64_t S, void *points, int32_t *n_valid,
+                                  void *bounds, const void *wires, int32_t W, int32_t ldw,
+                                  const int32_t *hit_offsets, const void *drift, uint8_t *hit_mask,
+                                  void *rss, int32_t *n_in, void *dca_out, int32_t *n_unconverged,
+                                  int64_t *idx_out, void *rss_out, uint8_t *hit_class, void *dca_wire,
+                                  int32_t update_mask, comet_stream stream);
 
 /* ---- a8/a9: classification (Sec. 2.1) and the mask of the next turn partition (Sec. 3.1) -------
  *   points, n_valid, charge, S, wires, W, ldw, hit_offsets, drift  as for comet_scan_dca.

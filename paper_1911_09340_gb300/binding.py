@@ -100,6 +100,9 @@ SIGNATURES = {
                                 C.POINTER(BatchCaps), C.POINTER(BatchEvent), _i32],
     "comet_scan_batch": [_vp, C.c_int, C.POINTER(_Field), C.POINTER(_Params), C.POINTER(BatchCaps),
                          C.POINTER(BatchEvent), _i32, _vp],
+    "comet_scan_partition": [_vp, C.c_int, C.POINTER(_Field), C.POINTER(_Params), C.POINTER(_Lattice),
+                             _i32, _vp, _vp, _i64, _vp, _vp, _vp, _vp, _i32, _i32, _vp, _vp, _vp, _vp,
+                             _vp, _vp, _vp, _vp, _vp, _vp, _vp, _i32, _vp],
     "comet_scan_classify": [_vp, C.c_int, C.POINTER(_Field), C.POINTER(_Params), _vp, _vp, _vp,
                             _i64, _vp, _vp, _i32, _i32, _vp, _vp, _vp, _vp, _vp, _i32, _vp],
 }
@@ -432,3 +435,21 @@ def comet_scan_classify(ctx: Context, field: DeviceField, params: ScanParams, po
                                      _ptr(hit_mask, torch.uint8), _ptr(hit_class, torch.uint8),
                                      _ptr(dca_wire, points.dtype), int(bool(update_mask)),
                                      _stream(stream)))
+
+
+def comet_scan_partition(ctx: Context, field: DeviceField, params: ScanParams, spec, k: int, seeds,
+                         charge, points, n_valid, bounds, wires, hit_offsets, drift, hit_mask, rss, n_in,
+                         idx, best, hit_class, dca_out=None, n_unconverged=None, dca_wire=None,
+                         update_mask: bool = False, n_wires: Optional[int] = None, stream=None):
+    """The arrays hold at least ``spec.n_seeds`` seeds (``points`` that many times 6 n_rec)."""
+    T = seeds.dtype
+    ldw = wires.shape[-1]
+    f, p, lat = field.c(), params.c(), lattice_struct(spec)
+    _check(lib().comet_scan_partition(
+        ctx.handle, _dtype_code(seeds), C.byref(f), C.byref(p), C.byref(lat), int(k), _ptr(seeds),
+        _ptr(charge, torch.int8), spec.n_seeds, _ptr(points, T), _ptr(n_valid, torch.int32),
+        _ptr(bounds, torch.float32), _ptr(wires, T), ldw if n_wires is None else int(n_wires), ldw,
+        _ptr(hit_offsets, torch.int32), _ptr(drift, T), _ptr(hit_mask, torch.uint8), _ptr(rss, T),
+        _ptr(n_in, torch.int32), _ptr(dca_out, T), _ptr(n_unconverged, torch.int32),
+        _ptr(idx, torch.int64), _ptr(best, T), _ptr(hit_class, torch.uint8), _ptr(dca_wire, T),
+        int(bool(update_mask)), _stream(stream)))

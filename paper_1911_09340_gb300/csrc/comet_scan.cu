@@ -836,4 +836,24 @@ comet_status comet_scan_classify(comet_ctx *ctx, comet_dtype dtype, const comet_
     return e == cudaSuccess ? COMET_OK : cuda_fail(e, "classify launch");
 }
 
+comet_status comet_scan_partition(comet_ctx *ctx, comet_dtype dtype, const comet_field *field,
+                                  const comet_scan_params *params, const comet_lattice *lat, int32_t k,
+                                  void *seeds, int8_t *charge, int64_t S, void *points, int32_t *n_valid,
+                                  void *bounds, const void *wires, int32_t W, int32_t ldw,
+                                  const int32_t *hit_offsets, const void *drift, uint8_t *hit_mask,
+                                  void *rss, int32_t *n_in, void *dca_out, int32_t *n_unconverged,
+                                  int64_t *idx_out, void *rss_out, uint8_t *hit_class, void *dca_wire,
+                                  int32_t update_mask, comet_stream stream)
+{
+    const bool fused = k == 1;
+    CHECK(comet_scan_lattice(ctx, dtype, lat, seeds, charge, S, stream));
+    CHECK(comet_scan_propagate(ctx, dtype, field, params, seeds, charge, S, points, n_valid, bounds, stream));
+    CHECK(comet_scan_dca(ctx, dtype, field, params, points, n_valid, charge, S, bounds, wires, W, ldw, hit_offsets,
+                         drift, hit_mask, rss, n_in, dca_out, n_unconverged, fused ? idx_out : nullptr,
+                         fused ? rss_out : nullptr, stream));
+    if (!fused) CHECK(comet_scan_select(ctx, dtype, rss, S, k, idx_out, rss_out, stream));
+    return comet_scan_classify(ctx, dtype, field, params, points, n_valid, charge, S, idx_out, wires, W, ldw,
+                               hit_offsets, drift, hit_mask, hit_class, dca_wire, update_mask, stream);
+}
+
 } // extern "C"

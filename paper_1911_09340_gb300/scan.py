@@ -74,6 +74,12 @@ class Workspace:
     def fits(self, S: int, n_rec: int, H: int) -> bool:
         return S <= self.S and n_rec <= self.n_rec and H <= self.hit_class.numel()
 
+    def holds(self, S: int, n_rec: int, k: int) -> bool:
+        """Whether the arrays, as they are, hold a partition of S seeds and its k best."""
+        return (1 <= k <= self.idx.numel() and k <= self.best.numel() and 6 * S <= self.seeds.numel()
+                and 6 * n_rec * S <= self.points.numel() and (S + 31) // 32 <= self.bounds.shape[0]
+                and S <= min(self.charge.numel(), self.n_valid.numel(), self.rss.numel(), self.n_in.numel()))
+
     def views(self, S: int, n_rec: int):
         """Contiguous views sized exactly for (S, n_rec)."""
         pts = self.points.view(-1)[: 6 * n_rec * S].view(6, n_rec, S)
@@ -97,6 +103,17 @@ def scan_partition(ctx: B.Context, field: B.DeviceField, params: B.ScanParams, s
     hit_class) and ``ev.mask`` (updated in place); with k = 1, ``best_idx`` / ``best_rss`` ([1]
     device tensors) take the selected seed and its RSS instead of ws.idx / ws.best."""
     S = spec.n_seeds
+    hc = ws.hit_class if hit_class is None else hit_class
+    if timer is None and ws.holds(S, params.n_rec, k) and hc.numel() >= max(ev.H, 1):
+        # the steps in one native call: five calls with their views cost 0.15 ms of host time, more than
+        # the kernels of a few hundred seeds
+        B.comet_scan_partition(
+            ctx, field, params, spec, k, ws.seeds, ws.charge, ws.points, ws.n_valid, ws.bounds, ev.wires,
+            ev.hit_offsets, ev.drift, ev.mask, ws.rss, ws.n_in,
+            ws.idx if k != 1 or best_idx is None else best_idx,
+            ws.best if k != 1 or best_rss is None else best_rss, hc, dca_out=want_dca,
+            n_unconverged=ws.n_unconv, dca_wire=dca_wire, update_mask=update_mask, n_wires=ev.W)
+        return ws
     seeds, charge, pts, nv, rss, n_in = ws.views(S, params.n_rec)
     mark = timer.mark if timer is not None else (lambda name: None)
     mark("lattice")

@@ -8,9 +8,9 @@ import torch
 
 import oracle as O
 from paper_1911_09340_gb300 import binding as B
-from paper_1911_09340_gb300 import synth
+from paper_1911_09340_gb300 import scan, synth
 
-from gpu_util import gpu_propagate
+from gpu_util import gpu_dca, gpu_propagate
 
 pytestmark = pytest.mark.gpu
 UNIFORM = synth.uniform_field(1.0)
@@ -122,3 +122,32 @@ def test_jacobian_lane_groups(ctx, n_seeds, n_wires, stride):
     assert np.allclose(srss.cpu(), (w * e * e + (1 - w) * lam * lam).sum(1), rtol=1e-12)
     assert np.allclose(jtr.cpu(), ((w * rho)[..., None] * J).sum(1), rtol=1e-10, atol=1e-12)
     assert np.allclose(jtj.cpu().numpy().reshape(-1, 4, 4), np.einsum("sw,swi,swj->sij", w, J, J), rtol=1e-10, atol=1e-12)
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.float64])
+@pytest.mark.parametrize("k,counts,want_dca", [(1, (2, 3, 4, 5), False), (1, (1, 1, 1, 1), True), (10, (3, 4, 5, 6), True),
+                                               (64, (4, 4, 4, 4), False)])
+def test_partition_in_one_call_equals_the_five(ctx, dtype, k, counts, want_dca):
+    """scan_partition without a timer is one native call, with one it is five: the same results, in a
+    workspace larger than the partition, with and without the optional outputs."""
+    ev = synth.multi_turn_event(1, counts=counts)
+    spec = ev.partitions[0]
+    bp = scan.event_params(ev, dtype, 16)[0]
+    out = []
+    for timer in (None, scan.KernelTimer()):
+        dev = scan.DeviceEvent.from_event(ev, dtype)
+        ws = scan.Workspace(spec.n_seeds + 40, bp.n_rec + 3, ev.n_hits + 5, dtype, k=k)
+        ws.hit_class.fill_(7)
+        dca = torch.full((dev.W, spec.n_seeds), -1.0, dtype=dtype, device="cuda") if want_dca else None
+        wire = torch.full((dev.W,), -1.0, dtype=dtype, device="cuda") if want_dca else None
+        best = torch.full((1,), -5, dtype=torch.int64, device="cuda") if k == 1 and want_dca else None
+        scan.scan_partition(ctx, B.DeviceField.from_synth(UNIFORM), bp, spec, dev, ws, k=k, want_dca=dca, dca_wire=wire,
+                            best_idx=best, timer=timer)
+        n = spec.n_seeds
+        out.append([ws.rss[:n], ws.n_in[:n], ws.idx if best is None else best, ws.best[:k], ws.hit_class, dev.mask,
+                    ws.n_unconv] + ([dca, wire] if want_dca else []))
+    for a, b in zip(*out):
+        assert torch.equal(a, b)
+    small = scan.Workspace(max(spec.n_seeds - 1, 1), bp.n_rec - 1, ev.n_hits, dtype, k=k)
+    with pytest.raises(RuntimeError):
+        scan.scan_partition(ctx, B.DeviceField.from_synth(UNIFORM), bp, spec, dev, small, k=k)
