@@ -526,13 +526,8 @@ __device__ __forceinline__ WireFrame<T> wire_frame(T ax, T ay, T az, T ux, T uy,
     return f;
 }
 
-// Distance form of the closest-state search (dca and classify use the same one, so that they pick the
-// same state): 1 = the wire frame (8 FP ops), 0 = the difference form line_dist2 (12 FP ops).
-#ifndef COMET_SEARCH_FRAME
-#define COMET_SEARCH_FRAME 1
-#endif
-
-// Squared distance of (x, y, z) to the wire line in the wire's frame.
+// Squared distance of (x, y, z) to the wire line in the wire's frame (dca and classify use this same
+// form, so that they pick the same state).
 template <typename T>
 __device__ __forceinline__ T frame_dist2(T x, T y, T z, T vx, T vy, T vz, T av, T wx, T wy, T wz,
                                          T aw)

@@ -18,13 +18,16 @@
 // recording kernel wrote (or built in shared memory when no table is given).  For each wire, the
 // lanes test the spheres in parallel (lane t: wire t against the super-segment spheres; then lane
 // m: level-1 sphere m of a candidate super-segment) and only segments whose bound does not exceed
-// the wire's capture radius (largest unmasked drift + lambda + h_rec/2) are scanned state by
-// state, each lane its own seed's states, keeping the lexicographic (distance, index) minimum.  If a seed's closest state is within the capture radius it lies in a
-// scanned segment, so the minimum is exact; if not, every residual of the wire is at least lambda
+// the wire's capture radius (largest unmasked drift + lambda + h_rec/2) are searched, each lane its own
+// seed's states, for the lexicographic (distance, index) minimum: runs of a few states are scanned state
+// by state, longer ones in an axial field walked down the valley of the distance (group_wires_long).
+// If a seed's closest state is within the capture radius it lies in a
+// searched segment, so the minimum is exact; if not, every residual of the wire is at least lambda
 // and the wire adds exactly lambda^2 to the RSS, with or without a refinement.  Beyond the first
 // and the last recorded state the refinement reaches up to h_rec (not h_rec/2) from the nearest
 // recorded state, so segments that may hold a track end are tested, and an end state refined,
-// within capture radius + h_rec.  With dca_out every state is scanned (exact DCA for every wire).
+// within capture radius + h_rec.  With dca_out (exact DCA for every wire) the spheres leave the segments
+// that may hold a lane's closest state; without a sphere table every state is then scanned.
 //
 // RSS: each thread sums its wires' d_i^2 in ascending wire order within each wire chunk (FP32 as a
 // TwoSum pair, FP64 plainly), then the chunks' sums in chunk order.  Atomics only hand out work
@@ -36,14 +39,19 @@
 #include "internal.h"
 
 // Tuning constants (compile-time): minimum resident CTAs per SM requested from the register
-// allocator, and how many states are loaded together.
+// allocator, and how many states are loaded together.  FP32 axial, short runs and every DCA: issue and
+// latency both count (8 CTAs: 2^18 x 70 states the same, 2^17 odd lattice 514 -> 547 us; 6: 469 us
+// against 452 at 2^18).  Long runs: 6 (2^14 x 2,229 states 157 us; 219 at 7, 227 at 8).
 #ifndef COMET_DCA_MINB
 #define COMET_DCA_MINB 7
 #endif
+#ifndef COMET_DCA_MINB_LONG
+#define COMET_DCA_MINB_LONG 6
+#endif
 // FP64: bound by the FP64 pipe rather than by resident warps; fewer CTAs per SM buy registers (at
-// 72 the FP64 kernels spill ~300 B per thread)
+// 72 the FP64 kernels spill ~300 B per thread; 4 CTAs 974 us, 3 CTAs 961 at 2^15 x 139 states)
 #ifndef COMET_DCA_MINB_F64
-#define COMET_DCA_MINB_F64 4
+#define COMET_DCA_MINB_F64 3
 #endif
 // FP32 in a non-axial field (tabulated or general uniform): RK4 stages in the refinement; at 72
 // registers the tabulated-field kernel spilled ~200 B per thread
@@ -52,11 +60,6 @@
 #endif
 #ifndef COMET_DCA_U2
 #define COMET_DCA_U2 2
-#endif
-// 1: the candidate scan loads each state's momentum with its position and keeps the closest
-// state, so that the refinement starts without a second dependent load
-#ifndef COMET_DCA_SCAN_P
-#define COMET_DCA_SCAN_P 1
 #endif
 // wires per chunk of the per-seed sums (the persistent kernel's finest work item)
 #ifndef COMET_DCA_CHUNK_W
@@ -136,7 +139,7 @@ struct Acc;
 template <>
 struct Acc<float> {
     float hi = 0.f, lo = 0.f;
-    __device__ __forceinline__ void add(float v) { two_sum_add(hi, lo, v); }
+    __device__ __forceinline__ void add_square(float d) { two_sum_add(hi, lo, __fmul_rn(d, d)); }
     __device__ __forceinline__ void add_pair(float h2, float l2)
     {
         two_sum_add(hi, lo, h2);
@@ -147,7 +150,7 @@ struct Acc<float> {
 template <>
 struct Acc<double> {
     double hi = 0.0, lo = 0.0;
-    __device__ __forceinline__ void add(double v) { hi += v; }
+    __device__ __forceinline__ void add_square(double d) { hi = fma(d, d, hi); }
     __device__ __forceinline__ void add_pair(double h2, double) { hi += h2; }
     __device__ __forceinline__ double value() const { return hi; }
 };
@@ -158,24 +161,9 @@ struct Acc<double> {
 // vectors and the offsets av = a.v, aw = a.w) and of the distance arithmetic moves the distance by
 // a few ulp of the coordinates involved, ~1e-7 m per metre of |av| + |aw| + reach; 2 um plus 1 um
 // per metre is a generous bound (the FP64 test it stands in for then never rejects more).
-__device__ __forceinline__ float sph_margin_f32(double av, double aw)
+__device__ __forceinline__ float sph_margin_f32(float av, float aw)
 {
-    return 2e-6f + 1e-6f * (float)(fabs(av) + fabs(aw));
-}
-
-template <typename T>
-__device__ __forceinline__ bool sphere_within(const float4 &sp, T fvx, T fvy, T fvz, T fav, T fwx,
-                                              T fwy, T fwz, T faw, T ax, T ay, T az, T ux, T uy,
-                                              T uz, T lim)
-{
-    if (sp.w < 0.f) return false;
-#if COMET_SEARCH_FRAME
-    const T d2 = frame_dist2<T>((T)sp.x, (T)sp.y, (T)sp.z, fvx, fvy, fvz, fav, fwx, fwy, fwz, faw);
-#else
-    const T d2 = line_dist2<T>((T)sp.x, (T)sp.y, (T)sp.z, ax, ay, az, ux, uy, uz);
-#endif
-    const T l = lim + (T)sp.w;
-    return d2 <= l * l;
+    return 2e-6f + 1e-6f * (fabsf(av) + fabsf(aw));
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -190,6 +178,7 @@ struct Group {
     int n0w;         // super-segments of the longest track of the warp
     int elo, ehi;    // smallest and largest last state index over the warp's tracks
     T c, ip;         // KAPPA q / P0, 1 / P0
+    float sz;        // |pz| / P0 (constant along the track in an axial field)
 };
 
 template <typename T>
@@ -204,10 +193,12 @@ __device__ __forceinline__ Group<T> load_group(const DcaArgs &a, int64_t g, int 
     gr.nv = 1;
     gr.c = T(0);
     gr.ip = T(0);
+    gr.sz = 0.f;
     if (gr.valid) {
         gr.nv = a.n_valid[gr.s];
-        seed_kinematics<T>(P[3 * plane + gr.s], P[4 * plane + gr.s], P[5 * plane + gr.s],
-                           a.charge[gr.s], gr.c, gr.ip);
+        const T pz = P[5 * plane + gr.s];
+        seed_kinematics<T>(P[3 * plane + gr.s], P[4 * plane + gr.s], pz, a.charge[gr.s], gr.c, gr.ip);
+        gr.sz = fabsf((float)(pz * gr.ip));
     }
     int n0w = gr.valid ? (gr.nv + a.G0 - 1) / a.G0 : 0;
 #pragma unroll
@@ -284,12 +275,43 @@ template <typename T>
 struct Tile {
     const T *ax, *ay, *az, *ux, *uy, *uz;   // wire point and direction, element i = wire w0 + i
     const Q4<T> *rec;                        // [wire][4]: (v, a.v), (w, a.w), (a, cap), (u, 0)
+    const float4 *ff;                        // FP64 only: [wire][2], (v, a.v) and (w, a.w) in float
     const T *cap;                            // capture radius (< 0: no unmasked hit)
     const int32_t *offs;                     // CSR offsets, element i = wire w0 + i
     const T *dsm;                            // drifts / masks: staged (global hit index) or global
     const uint8_t *msm;
     int w0, wn;
 };
+
+// Wire i's frame (v, a.v), (w, a.w) for the sphere tests, which are made in float in either precision:
+// the part's FP64 rate would be the limit there, and an FP64 tile keeps a float copy of its frames.
+template <typename T>
+__device__ __forceinline__ void sphere_frame(const Tile<T> &tl, int i, float4 &v, float4 &w)
+{
+    if constexpr (sizeof(T) == 4) {
+        const Q4<T> a = tl.rec[4 * i + 0], b = tl.rec[4 * i + 1];
+        v = make_float4(a.x, a.y, a.z, a.w);
+        w = make_float4(b.x, b.y, b.z, b.w);
+    } else {
+        v = tl.ff[2 * i + 0];
+        w = tl.ff[2 * i + 1];
+    }
+}
+
+// Extra reach of a sphere test of the FP64 kernels (none in FP32, whose margins are in the spheres).
+template <typename T>
+__device__ __forceinline__ float sphere_margin(float av, float aw)
+{
+    return sizeof(T) == 4 ? 0.f : sph_margin_f32(av, aw);
+}
+
+// Whether the sphere reaches within lim of the wire; d2 = the squared distance of its centre.
+__device__ __forceinline__ bool sphere_within(const float4 &sp, const float4 &v, const float4 &w, float lim, float &d2)
+{
+    d2 = frame_dist2<float>(sp.x, sp.y, sp.z, v.x, v.y, v.z, v.w, w.x, w.y, w.z, w.w);
+    const float l = lim + sp.w;
+    return sp.w >= 0.f && d2 <= l * l;
+}
 
 // Capture radius and frame of wire i of a staged tile (one thread per wire), packed with its
 // point and direction into the wire's four records.
@@ -310,17 +332,292 @@ __device__ __forceinline__ void tile_wire_setup(const Tile<T> &tl, int i, T lam,
     rec[4 * i + 3] = Q4<T>{ux, uy, uz, T(0)};
 }
 
-// Wires [wb, we) of one tile for one 32-seed group: accumulates d_i^2, n_in and unconverged counts.
+// The float copies of an FP64 tile's frames, in the shared memory of its staged rows (read for the last
+// time by tile_wire_setup: the caller's barrier lies between).
+template <typename T>
+__device__ __forceinline__ void tile_float_frames(const Q4<T> *rec, int wn, float4 *ff)
+{
+    if constexpr (sizeof(T) == 8)
+        for (int i = threadIdx.x; i < 2 * wn; i += blockDim.x) {
+            const Q4<T> r = rec[4 * (i >> 1) + (i & 1)];
+            ff[i] = make_float4((float)r.x, (float)r.y, (float)r.z, (float)r.w);
+        }
+}
+
+// Tighter reach of the refinement from an interior closest state (axial field): at a point of
+// closest approach X* with distance D, the recorded state within delta <= h_rec/2 of it along the
+// track is at most sqrt(D^2 + delta^2) + kappa delta^2 / 2 from the wire (the tangent line from
+// X* moves away from the wire as sqrt(D^2 + delta^2 |t_perp|^2), the track leaves the tangent by
+// at most kappa delta^2 / 2, kappa = |KAPPA q B / P0| its curvature).  So a closest recorded state
+// farther than sqrt(cap^2 + (h_rec/2)^2) + kappa (h_rec/2)^2 / 2 cannot refine to D < cap: the
+// wire adds lambda^2.  Returned: the warp's largest kappa times (h_rec/2)^2 / 2, plus the margin
+// (infinite in other fields).
 template <typename T, class F>
-__device__ __forceinline__ void group_wires(const F &f, const DcaArgs &a, const Group<T> &gr,
+__device__ __forceinline__ T warp_curvature(const F &f, const Group<T> &gr)
+{
+    T kap = T(0);
+    if constexpr (F::kAxial) {
+        kap = fabs(gr.c * f.bz);
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) kap = fmax(kap, __shfl_xor_sync(0xffffffffu, kap, off));
+    }
+    return kap;
+}
+
+template <typename T, class F>
+__device__ __forceinline__ T interior_margin(const F &f, const DcaArgs &a, const Group<T> &gr)
+{
+    if constexpr (!F::kAxial) return T(INFINITY);
+    const T half_rec = in_prec<T>(a.half_rec, a.half_rec_f);
+    return T(0.5) * warp_curvature<T, F>(f, gr) * half_rec * half_rec + in_prec<T>(a.margin, a.margin_f);
+}
+
+// First refinement step, to the vertex of the parabola through the squared distances of the
+// closest state and its two neighbours (exact for a straight track, where the squared distance is
+// quadratic in arc length); then Newton steps as usual.  0 (none) unless both neighbours were
+// looked at and the step budget allows (max_iter >= 4).
+template <typename T>
+__device__ __forceinline__ T first_step(const DcaArgs &a, T h_rec, T bdm, T bd, T bdp)
+{
+    T s0 = T(0);
+    if (a.max_iter >= 4 && bdm < T(INFINITY) && bdp < T(INFINITY)) {
+        const T den = bdm - T(2) * bd + bdp;
+        if (den > T(0)) {
+            s0 = T(0.5) * h_rec * (bdm - bdp) / den;
+            s0 = fmin(fmax(s0, -h_rec), h_rec);
+        }
+    }
+    return s0;
+}
+
+// Whether a wire has an unmasked hit (capture radius not negative; the sign bit, off the FP64 pipe).
+template <typename T>
+__device__ __forceinline__ bool has_hit(T cap)
+{
+    if constexpr (sizeof(T) == 4)
+        return cap >= T(0);
+    else
+        return __double2hiint(cap) >= 0;
+}
+
+// Whether the squared distance a is below b (both not negative; as integers, which order alike and spare
+// the FP64 pipe a comparison).  A NaN is below nothing.
+template <typename T>
+__device__ __forceinline__ bool nearer(T a, T b)
+{
+    if constexpr (sizeof(T) == 4)
+        return a < b;
+    else
+        return (unsigned long long)__double_as_longlong(a) < (unsigned long long)__double_as_longlong(b);
+}
+
+// Wire ii's residual of Eq. 1 for a refined seed: the smallest |D - r| over its unmasked hits, capped at
+// lambda (below lambda it counts into n_in).
+template <typename T>
+__device__ __forceinline__ T residual(const Tile<T> &tl, int ii, T D, T lam, int &nin)
+{
+    T emin = T(INFINITY);
+    const int hb = tl.offs[ii], he = tl.offs[ii + 1];
+    for (int j = hb; j < he; ++j) {
+        if (tl.msm[j]) continue;
+        const T e = fabs(D - tl.dsm[j]);
+        if (nearer<T>(e, emin)) emin = e;
+    }
+    if (!nearer<T>(emin, lam)) return lam;
+    ++nin;
+    return emin;
+}
+
+// Shorter runs are scanned one state after the other with its momentum, longer ones two positions at a
+// time and the momentum of the closest state loaded at the end (group_wires_short).  Recordings of 32 mm
+// give runs of 1.5 states, of 16 mm up to 13 (an odd lattice's wide groups): 2^18 x 70 states 445 us
+// in pairs with momentum, 449 us so; 76,545 x 139 (odd lattice) 569 and 514 us, all one by one 675 us.
+constexpr int kFewStates = 4;
+
+// Runs of more than this many states are walked, not scanned (group_wires_long): a walk looks at about
+// four states, costs as much as ten in FP32 (less in FP64, where distances are dear).
+template <typename T>
+constexpr int kWalkMin = sizeof(T) == 4 ? 10 : 4;
+
+// Wires [wb, we) of one tile for one 32-seed group: accumulates d_i^2, n_in and unconverged counts.  Two
+// forms with the same results.  SHORT: runs of a few candidate states (one-state segments), each scanned
+// with its momentum loaded beside its position, so that the refinement starts without another round trip
+// to memory (with few warps resident, latency counts as much as issue).  Otherwise group_wires_long:
+// positions only, runs of many states walked, and the search bounded by the spheres when every DCA
+// is wanted.  Both are bound by instruction issue (72% of it used at 2^18 seeds), the refinement taking
+// the larger part.  Before (one form, 64-bit addresses, momentum selected along) and after, FP32: 2^18 seeds
+// x 70 states 463 -> 449 us, 76,545 x 139 592 -> 514, 2^14 x 2,229 560 -> 157, every DCA of 2^14 x 70
+// 373 -> 101; FP64: 4,096 x 2,229 808 -> 280, 2^15 x 139 1415 -> 1250.
+// Off: the byte offset of a recorded value, 32 bits when the track array is small enough.
+template <typename T, class F, typename Off>
+__device__ __forceinline__ void group_wires_short(const F &f, const DcaArgs &a, const Group<T> &gr,
+                                                  const Tile<T> &tl, const float4 *sph0,
+                                                  const float4 *sph1, int lane, Acc<T> &acc, int &nin,
+                                                  int &nunc, int wb, int we)
+{
+    const int64_t S = a.S;
+    const int64_t s = gr.s;
+    const char *__restrict__ pts = (const char *)a.points;
+    const Off row = (Off)S * (Off)sizeof(T), col = (Off)s * (Off)sizeof(T), plane = (Off)a.n_rec * row;
+    auto val = [=](int c, Off o) { return *(const T *)(pts + (Off)(o + (Off)c * plane)); };
+    const bool valid = gr.valid;
+    const int nv = gr.nv;
+    const T lam = in_prec<T>(a.lambda, a.lambda_f), tol = in_prec<T>(a.tol, a.tol_f),
+            half_rec = in_prec<T>(a.half_rec, a.half_rec_f), h_rec = in_prec<T>(a.h_rec, a.h_rec_f);
+    const int G0 = a.G0, G1 = a.G1;
+    const int N1 = (G0 + G1 - 1) / G1;
+    const Q4<T> *rec = tl.rec;
+    const T kq2 = interior_margin<T, F>(f, a, gr);
+    const T hq2 = half_rec * half_rec;
+
+    for (int base = wb; base < we; base += 32) {
+        const int clen = min(32, we - base);
+        // lane t: which super-segments can bring wire base + t within its capture radius, and the wire's
+        // interior reach
+        uint32_t mask0 = 0;
+        T thin_t = T(0);
+        if (lane < clen) {
+            const int iw = base + lane;
+            const T capw = tl.cap[iw];
+            if (capw >= T(0)) {
+                float4 q0, q1;
+                sphere_frame<T>(tl, iw, q0, q1);
+                const float l = (float)(capw + half_rec) + sphere_margin<T>(q0.w, q1.w);
+                for (int j = 0; j < gr.n0w; ++j) {
+                    float d2;
+                    if (sphere_within(sph0[j], q0, q1, l, d2)) mask0 |= 1u << j;
+                }
+                thin_t = fmin(capw + half_rec, sqrt(capw * capw + hq2) + kq2);
+            }
+        }
+        for (int t = 0; t < clen; ++t) {
+            const int ii = base + t;
+            const uint32_t m0 = __shfl_sync(0xffffffffu, mask0, t);
+            const Q4<T> r2 = rec[4 * ii + 2];
+            const T cap = r2.w;
+            const bool used = valid && has_hit<T>(cap);
+            if (m0 == 0u) {
+                // beyond every seed's capture radius (or no unmasked hit): lambda^2 if in the sum
+                if (used) acc.add_square(lam);
+                continue;
+            }
+            const T thin = __shfl_sync(0xffffffffu, thin_t, t);
+            const Q4<T> r0 = rec[4 * ii + 0], r1 = rec[4 * ii + 1];
+            const T capth = cap + half_rec;
+            // the closest state so far, loaded with the scan (no second round trip to refine), and the
+            // squared distances of the states scanned just before and after it (for the first
+            // refinement step); the state scanned last: its distance, and whether it is the closest
+            T bd = T(INFINITY), bdm = T(INFINITY), bdp = T(INFINITY), dprev = T(INFINITY);
+            T by[6] = {T(0), T(0), T(0), T(0), T(0), T(0)};
+            int bk = 0x7fffffff, kend = -1;
+            bool last = false;
+            float4 q0, q1;
+            sphere_frame<T>(tl, ii, q0, q1);
+            const float mg = sphere_margin<T>(q0.w, q1.w);
+            uint32_t u0 = m0;
+            while (u0) {
+                const int j = __ffs(u0) - 1;
+                u0 &= u0 - 1;
+                // lane m tests level-1 segment m of super-segment j; a one-state segment
+                // that may hold a track end (the first state, or between the warp's smallest
+                // and largest last state) gets the refinement's extra half interval there;
+                // one-state segments away from the track ends need only the interior reach
+                const int k1 = j * G0 + lane;
+                const bool end1 = G1 == 1 && (k1 == 0 || (k1 >= gr.elo && k1 <= gr.ehi));
+                const float lim1 = (float)(G1 == 1 ? (end1 ? capth + half_rec : thin) : capth) + mg;
+                float d2;
+                const uint32_t u1 = __ballot_sync(0xffffffffu, lane < N1 && sphere_within(sph1[j * kN1Max + lane], q0, q1, lim1, d2));
+                if (u1) {
+                    // one contiguous range from the first to the last candidate level-1 segment (a
+                    // superset of the candidates; their loads go out together), kU states at a time;
+                    // ranges come in ascending order, so an equal distance never replaces the one found
+                    const int k0 = j * G0 + (__ffs(u1) - 1) * G1;
+                    const int ke = min(j * G0 + (32 - __clz(u1)) * G1, j * G0 + G0);
+                    const int kv = used ? min(ke, nv) : 0;
+                    if (k0 != kend) {
+                        dprev = T(INFINITY);
+                        last = false;
+                    }
+                    kend = ke;
+                    auto dist = [&](T x, T y, T z) {
+                        return frame_dist2<T>(x, y, z, r0.x, r0.y, r0.z, r0.w, r1.x, r1.y, r1.z, r1.w);
+                    };
+                    auto look = [&](int k, T d) {   // the next state's distance; whether it is the closest
+                        const bool now = nearer<T>(d, bd);
+                        if (last) bdp = d;
+                        if (now) {
+                            bdm = dprev;
+                            bdp = T(INFINITY);
+                            bd = d;
+                            bk = k;
+                        }
+                        dprev = d;
+                        last = now;
+                        return now;
+                    };
+                    Off o = (Off)k0 * row + col;
+                    if (ke - k0 < kFewStates) {
+                        for (int k = k0; k < ke; ++k, o += row)
+                            if (k < kv) {
+                                T x[6];
+#pragma unroll
+                                for (int c = 0; c < 6; ++c) x[c] = val(c, o);
+                                if (look(k, dist(x[0], x[1], x[2])))
+#pragma unroll
+                                    for (int c = 0; c < 6; ++c) by[c] = x[c];
+                            }
+                    } else {
+                        const int before = bk;
+                        for (int k = k0; k < ke; k += 2, o += 2 * row) {
+                            T xa[3], xb[3];
+                            if (k < kv)
+#pragma unroll
+                                for (int c = 0; c < 3; ++c) xa[c] = val(c, o);
+                            if (k + 1 < kv)
+#pragma unroll
+                                for (int c = 0; c < 3; ++c) xb[c] = val(c, o + row);
+                            if (k < kv) look(k, dist(xa[0], xa[1], xa[2]));
+                            if (k + 1 < kv) look(k + 1, dist(xb[0], xb[1], xb[2]));
+                        }
+                        if (bk != before) {
+                            o = (Off)bk * row + col;
+#pragma unroll
+                            for (int c = 0; c < 6; ++c) by[c] = val(c, o);
+                        }
+                    }
+                }
+            }
+
+            // refinement from the closest recorded state, only where it can bring the wire within
+            // its capture radius (group_wires_long)
+            const T th = (bk == 0 || bk == nv - 1) ? capth + half_rec : thin;
+            const bool refine = bk != 0x7fffffff && bd <= th * th;
+            T d = lam;   // lambda when the wire is not refined
+            if (refine) {
+                T D;
+                const Q4<T> r3 = rec[4 * ii + 3];
+                const T s0 = first_step<T>(a, h_rec, bdm, bd, bdp);
+                const int conv = refine_dca<T, F>(f, gr.c, gr.ip, by, r2.x, r2.y, r2.z, r3.x, r3.y, r3.z, tol,
+                                                  a.max_iter, h_rec, D, s0);
+                nunc += 1 - conv;
+                d = residual<T>(tl, ii, D, lam, nin);
+            }
+            if (used) acc.add_square(d);
+        }
+    }
+}
+
+template <typename T, class F, typename Off, bool ALL>
+__device__ __forceinline__ void group_wires_long(const F &f, const DcaArgs &a, const Group<T> &gr,
                                             const Tile<T> &tl, const float4 *sph0,
                                             const float4 *sph1, int lane, Acc<T> &acc, int &nin,
                                             int &nunc, int wb, int we)
 {
-    const T *__restrict__ P = (const T *)a.points;
     const int64_t S = a.S;
-    const int64_t plane = (int64_t)a.n_rec * S;
     const int64_t s = gr.s;
+    const char *__restrict__ pts = (const char *)a.points;
+    const Off row = (Off)S * (Off)sizeof(T), col = (Off)s * (Off)sizeof(T), plane = (Off)a.n_rec * row;
+    auto val = [=](int c, Off o) { return *(const T *)(pts + (Off)(o + (Off)c * plane)); };
     const bool valid = gr.valid;
     const int nv = gr.nv;
     const T lam = in_prec<T>(a.lambda, a.lambda_f), tol = in_prec<T>(a.tol, a.tol_f),
@@ -329,185 +626,229 @@ __device__ __forceinline__ void group_wires(const F &f, const DcaArgs &a, const 
     const int N1 = (G0 + G1 - 1) / G1;
     const Q4<T> *rec = tl.rec;
     constexpr int kU = COMET_DCA_U2;
-    // Tighter reach of the refinement from an interior closest state (axial field): at a point of
-    // closest approach X* with distance D, the recorded state within delta <= h_rec/2 of it along the
-    // track is at most sqrt(D^2 + delta^2) + kappa delta^2 / 2 from the wire (the tangent line from
-    // X* moves away from the wire as sqrt(D^2 + delta^2 |t_perp|^2), the track leaves the tangent by
-    // at most kappa delta^2 / 2, kappa = |KAPPA q B / P0| its curvature).  So a closest recorded state
-    // farther than sqrt(cap^2 + (h_rec/2)^2) + kappa (h_rec/2)^2 / 2 cannot refine to D < cap: the
-    // wire adds lambda^2.  kq2 = the warp's largest kappa times (h_rec/2)^2 / 2, plus the margin.
-    T kq2 = T(INFINITY);
+    const T kq2 = interior_margin<T, F>(f, a, gr);
+    // for the walk to the closest state (see below)
+    [[maybe_unused]] float szw = 0.f, dcv_k = 0.f, hg_k = 0.f;
     if constexpr (F::kAxial) {
-        T kap = fabs(gr.c * f.bz);
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) kap = fmax(kap, __shfl_xor_sync(0xffffffffu, kap, off));
-        kq2 = T(0.5) * kap * half_rec * half_rec + in_prec<T>(a.margin, a.margin_f);
+        szw = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(gr.sz)));
+        const float kf = fmaxf((float)warp_curvature<T, F>(f, gr), 1e-6f);
+        dcv_k = 0.8f / kf;
+        hg_k = 0.25f * kf * a.h_rec_f * a.h_rec_f;
     }
     const T hq2 = half_rec * half_rec;
+    const bool pruned = !ALL || sph0 != nullptr;   // no spheres: every state is scanned (dca_out without bounds)
 
     for (int base = wb; base < we; base += 32) {
         const int clen = min(32, we - base);
         // lane t: which super-segments can bring wire base + t within its capture radius
         uint32_t mask0 = 0;
+        T thin_t = T(INFINITY);   // interior reach (see interior_margin), never above cap + half_rec
+        [[maybe_unused]] float dcv_t = 0.f;   // distance below which wire base + t's valley is convex
         if (lane < clen) {
             const int iw = base + lane;
             const T capw = tl.cap[iw];
-            if (a.exact_all) {
-                mask0 = 1u;
+            if constexpr (F::kAxial) {
+                const float uzf = fabsf((float)rec[4 * iw + 3].z);
+                const float tau = szw * uzf + sqrtf(fmaxf(1.f - uzf * uzf, 0.f)) + 1e-3f;
+                const float conv = 1.f - tau * tau;
+                dcv_t = conv > 0.05f ? conv * dcv_k : 0.f;
+            }
+            if (ALL) {
+                mask0 = (1u << gr.n0w) - 1u;
             } else if (capw >= T(0)) {
-                const T lim = capw + half_rec;
-                const Q4<T> r0 = rec[4 * iw + 0], r1 = rec[4 * iw + 1], r2 = rec[4 * iw + 2],
-                            r3 = rec[4 * iw + 3];
-                if constexpr (sizeof(T) == 8) {
-                    // FP64 kernels test the (float) spheres in FP32: the part's FP64 rate is the
-                    // limit there.  The reach grows by sph_margin_f32 so that the test stays a
-                    // superset of the FP64 one.
-                    const float l = (float)lim + sph_margin_f32(r0.w, r1.w);
-                    const float v0 = (float)r0.x, v1 = (float)r0.y, v2 = (float)r0.z, va = (float)r0.w;
-                    const float w0 = (float)r1.x, w1 = (float)r1.y, w2 = (float)r1.z, wa = (float)r1.w;
-                    for (int j = 0; j < gr.n0w; ++j)
-                        if (sphere_within<float>(sph0[j], v0, v1, v2, va, w0, w1, w2, wa, (float)r2.x,
-                                                 (float)r2.y, (float)r2.z, (float)r3.x, (float)r3.y,
-                                                 (float)r3.z, l))
-                            mask0 |= 1u << j;
-                } else {
-                    for (int j = 0; j < gr.n0w; ++j)
-                        if (sphere_within<T>(sph0[j], r0.x, r0.y, r0.z, r0.w, r1.x, r1.y, r1.z, r1.w,
-                                             r2.x, r2.y, r2.z, r3.x, r3.y, r3.z, lim))
-                            mask0 |= 1u << j;
+                thin_t = fmin(capw + half_rec, sqrt(capw * capw + hq2) + kq2);
+                float4 q0, q1;
+                sphere_frame<T>(tl, iw, q0, q1);
+                const float l = (float)(capw + half_rec) + sphere_margin<T>(q0.w, q1.w);
+                for (int j = 0; j < gr.n0w; ++j) {
+                    float d2;
+                    if (sphere_within(sph0[j], q0, q1, l, d2)) mask0 |= 1u << j;
                 }
             }
         }
         for (int t = 0; t < clen; ++t) {
             const int ii = base + t;
             const uint32_t m0 = __shfl_sync(0xffffffffu, mask0, t);
+            [[maybe_unused]] const float dcv = F::kAxial ? __shfl_sync(0xffffffffu, dcv_t, t) : 0.f;
             const Q4<T> r2 = rec[4 * ii + 2];
             const T cap = r2.w;
+            const bool used = valid && has_hit<T>(cap);
             if (m0 == 0u) {
                 // beyond every seed's capture radius (or no unmasked hit): lambda^2 if in the sum
-                if (valid && cap >= T(0)) acc.add(lam * lam);
+                if (used) acc.add_square(lam);
                 continue;
             }
-            const Q4<T> r0 = rec[4 * ii + 0], r1 = rec[4 * ii + 1], r3 = rec[4 * ii + 3];
-            const T ax = r2.x, ay = r2.y, az = r2.z;
-            const T ux = r3.x, uy = r3.y, uz = r3.z;
-            const T fvx = r0.x, fvy = r0.y, fvz = r0.z, fav = r0.w;
-            const T fwx = r1.x, fwy = r1.y, fwz = r1.z, faw = r1.w;
-#if COMET_SEARCH_FRAME
-            auto sd2 = [&](T x, T y, T z) {
-                return frame_dist2<T>(x, y, z, fvx, fvy, fvz, fav, fwx, fwy, fwz, faw);
-            };
-#else
-            auto sd2 = [&](T x, T y, T z) { return line_dist2<T>(x, y, z, ax, ay, az, ux, uy, uz); };
-#endif
-            const bool want = valid && (cap >= T(0) || a.exact_all);
-            const T capth = a.exact_all ? T(INFINITY) : cap + half_rec;
-            // interior reach (see kq2): never above capth
-            const T thin = a.exact_all ? T(INFINITY) : fmin(capth, sqrt(cap * cap + hq2) + kq2);
-            T bd = T(INFINITY);
+            const Q4<T> r0 = rec[4 * ii + 0], r1 = rec[4 * ii + 1];
+            const T thin = __shfl_sync(0xffffffffu, thin_t, t);
+            const bool want = used || (valid && ALL);
+            const T capth = ALL ? T(INFINITY) : cap + half_rec;
+            // the closest state so far, and the squared distances of the states before and after it
+            // (for the first refinement step; infinite where there is none or it was not looked at)
+            T bd = T(INFINITY), bdm = T(INFINITY), bdp = T(INFINITY);
             int bk = 0x7fffffff;
-#if COMET_DCA_SCAN_P
-            // the closest state so far, loaded with the scan (no second round trip to refine)
-            T by[6] = {T(0), T(0), T(0), T(0), T(0), T(0)};
-            // squared distances of the states scanned just before and after the closest one (for
-            // the first refinement step) and of the previous state scanned
-            T bdm = T(INFINITY), bdp = T(INFINITY), dprev = T(INFINITY);
-            int kprev = -2;
-#endif
-            // scans states [k0, k1) of this lane's seed, kU at a time (span is warp-uniform)
+            auto dist_at = [&](Off o) {
+                return frame_dist2<T>(val(0, o), val(1, o), val(2, o), r0.x, r0.y, r0.z, r0.w, r1.x, r1.y, r1.z, r1.w);
+            };
+            // every state of [k0, k1) of this lane's seed, kU at a time (span is warp-uniform); ranges come in
+            // ascending order, so an equal distance never replaces the one found
             auto scan = [&](int k0, int k1, int span) {
-                // one 64-bit multiply per range; states are S elements apart
-                const T *q0 = P + ((int64_t)k0 * S + s);
-                for (int t0 = 0; t0 < span; t0 += kU, q0 += kU * S) {
-                    T xs[kU], ys[kU], zs[kU];
-#if COMET_DCA_SCAN_P
-                    T pxs[kU], pys[kU], pzs[kU];
-#endif
+                Off o = (Off)k0 * row + col;
+                T dprev = T(INFINITY);
+                bool last = false;   // the previous state is the closest so far
+                k1 = want ? k1 : 0;
+                for (int t0 = 0; t0 < span; t0 += kU, o += kU * row) {
+                    T d[kU];
+#pragma unroll
+                    for (int u = 0; u < kU; ++u) d[u] = k0 + t0 + u < k1 ? dist_at(o + u * row) : T(INFINITY);
 #pragma unroll
                     for (int u = 0; u < kU; ++u) {
-                        const int k = k0 + t0 + u;
-                        xs[u] = ys[u] = zs[u] = T(0);
-#if COMET_DCA_SCAN_P
-                        pxs[u] = pys[u] = pzs[u] = T(0);
-#endif
-                        if (want && k < k1) {
-                            const T *q = q0 + u * S;
-                            xs[u] = q[0];
-                            ys[u] = q[plane];
-                            zs[u] = q[2 * plane];
-#if COMET_DCA_SCAN_P
-                            pxs[u] = q[3 * plane];
-                            pys[u] = q[4 * plane];
-                            pzs[u] = q[5 * plane];
-#endif
+                        const bool now = nearer<T>(d[u], bd);
+                        bdp = now ? T(INFINITY) : (last ? d[u] : bdp);
+                        if (now) {
+                            bdm = dprev;
+                            bd = d[u];
+                            bk = k0 + t0 + u;
                         }
-                    }
-#pragma unroll
-                    for (int u = 0; u < kU; ++u) {
-                        const int k = k0 + t0 + u;
-                        if (want && k < k1) {
-#if COMET_DCA_SCAN_P
-                            const T d = sd2(xs[u], ys[u], zs[u]);
-                            if (d < bd || (d == bd && k < bk)) {
-                                bdm = k == kprev + 1 ? dprev : T(INFINITY);
-                                bdp = T(INFINITY);
-                                bd = d;
-                                bk = k;
-                                by[0] = xs[u];
-                                by[1] = ys[u];
-                                by[2] = zs[u];
-                                by[3] = pxs[u];
-                                by[4] = pys[u];
-                                by[5] = pzs[u];
-                            } else if (k == bk + 1) {
-                                bdp = d;
-                            }
-                            dprev = d;
-                            kprev = k;
-#else
-                            lex_min<T>(bd, bk, sd2(xs[u], ys[u], zs[u]), k);
-#endif
-                        }
+                        dprev = d[u];
+                        last = now;
                     }
                 }
             };
-            if (a.exact_all) {
-                int nvw = nv;
-#pragma unroll
-                for (int off = 16; off > 0; off >>= 1) nvw = max(nvw, __shfl_xor_sync(0xffffffffu, nvw, off));
-                scan(0, nv, nvw);
+            // The closest state of a run [ra, rb] of candidate states.  Axial field: down the valley from a
+            // start state, without scanning it.  Along a track f = d^2 / 2 has f'' = |t_perp|^2 + e . dt/ds
+            // >= 1 - (t.u)^2 - kappa d, and |t.u| <= |tz uz| + sqrt(1 - uz^2) (tz = pz / P0 is constant), so
+            // f'' >= 0.2 (1 - tau^2) wherever d <= dcv = 0.8 (1 - tau^2) / kappa.  Where that holds for the
+            // whole run (its states lie at most their arc length farther than the state found), a state
+            // with no closer neighbour is its closest.  Rounding: two states beyond the found one d^2 has
+            // grown by 0.4 (1 - tau^2) h^2, which hg requires to be above 16 d times an eighth of the search
+            // margin, the rounding of a distance.  A warp with a lane that does not meet this, or that is
+            // not there after kSteps moves, scans the run.
+            // The neighbours' distances are handed on where a scan of the run would have them, so both ways
+            // give the same bits.
+            auto closest_in = [&](int ra, int rb, int kst) {
+                const int side = ALL ? 1 : 0;   // a scan of every state knows all neighbours
+                if constexpr (F::kAxial)
+                    if (rb - ra >= kWalkMin<T>) {
+                        bool ok = true;
+                        T d0 = T(INFINITY), dm = T(INFINITY), dp = T(INFINITY);
+                        int k = 0;
+                        if (want) {
+                            k = min(kst, nv - 1);
+                            if (G1 > 1) {
+                                // the start is a segment's centre, several states from this lane's closest:
+                                // one Newton step of d^2 along the track's tangent, in whole states
+                                float4 v, w;
+                                sphere_frame<T>(tl, ii, v, w);
+                                const Off o = (Off)k * row + col;
+                                const float x = (float)val(0, o), y = (float)val(1, o), z = (float)val(2, o);
+                                const float px = (float)val(3, o), py = (float)val(4, o), pz = (float)val(5, o);
+                                const float ev = fmaf(x, v.x, fmaf(y, v.y, fmaf(z, v.z, -v.w)));
+                                const float ew = fmaf(x, w.x, fmaf(y, w.y, fmaf(z, w.z, -w.w)));
+                                const float pv = px * v.x + py * v.y + pz * v.z, pw = px * w.x + py * w.y + pz * w.z;
+                                const float n = __fdividef(-(ev * pv + ew * pw),
+                                                           (pv * pv + pw * pw) * (float)gr.ip * a.h_rec_f);
+                                k = max(0, min(k + (int)rintf(fminf(fmaxf(n, -256.f), 256.f)), nv - 1));
+                            }
+                            Off o = (Off)k * row + col;
+                            d0 = dist_at(o);
+                            if (k > 0) dm = dist_at(o - row);
+                            if (k < nv - 1) dp = dist_at(o + row);
+                            constexpr int kSteps = 6;
+                            for (int it = 0; it < kSteps && (dm <= d0 || dp < d0); ++it) {
+                                if (dm <= d0) {
+                                    --k;
+                                    o -= row;
+                                    dp = d0;
+                                    d0 = dm;
+                                    dm = k > 0 ? dist_at(o - row) : T(INFINITY);
+                                } else {
+                                    ++k;
+                                    o += row;
+                                    dm = d0;
+                                    d0 = dp;
+                                    dp = k < nv - 1 ? dist_at(o + row) : T(INFINITY);
+                                }
+                            }
+                            const float far = dcv - a.h_rec_f * (float)(1 + max(0, max(k - min(ra, nv - 1), min(rb, nv - 1) - k)));
+                            const float hg = hg_k * dcv, f0 = (float)d0;
+                            ok = !(dm <= d0 || dp < d0) && far > 0.f && f0 <= far * far &&
+                                 f0 * (a.margin_f * a.margin_f) <= hg * hg;
+                        }
+                        if (__all_sync(0xffffffffu, ok)) {
+                            if (want && (d0 < bd || (d0 == bd && k < bk))) {
+                                bd = d0;
+                                bk = k;
+                                bdm = k > ra - side ? dm : T(INFINITY);
+                                bdp = k < rb + side ? dp : T(INFINITY);
+                            }
+                            return;
+                        }
+                    }
+                const int k0 = max(ra - side, 0);
+                scan(k0, min(rb + 1 + side, nv), rb + 1 + side - k0);
+            };
+            if (!pruned) {
+                scan(0, nv, gr.ehi + 1);
             } else {
+                float4 q0, q1;
+                sphere_frame<T>(tl, ii, q0, q1);
+                const float mg = sphere_margin<T>(q0.w, q1.w);
+                float lim_end = (float)(capth + half_rec) + mg, lim_in = (float)(G1 == 1 ? thin : capth) + mg;
+                if (ALL) {
+                    // no state of any lane's closest is farther than the nearest sphere that all lanes have
+                    // reaches: spheres beyond it hold no closest state
+                    float ub = INFINITY;
+                    for (int j = 0; j < gr.n0w; ++j) {
+                        const float4 sp = lane < N1 ? sph1[j * kN1Max + lane] : make_float4(0.f, 0.f, 0.f, -1.f);
+                        float d2;
+                        if (j * G0 + lane * G1 <= gr.elo && sphere_within(sp, q0, q1, INFINITY, d2))
+                            ub = fminf(ub, sqrtf(d2) + sp.w);
+                    }
+                    lim_in = lim_end = __uint_as_float(__reduce_min_sync(0xffffffffu, __float_as_uint(ub))) +
+                                       a.margin_f + 2.f * mg;
+                }
+                // Runs of candidate level-1 segments, super-segment by super-segment (lane m tests segment
+                // m); a run that goes on into the next super-segment is one run.
                 uint32_t u0 = m0;
-                while (u0) {
-                    const int j = __ffs(u0) - 1;
-                    u0 &= u0 - 1;
-                    // lane m tests level-1 segment m of super-segment j; a one-state segment
-                    // that may hold a track end (the first state, or between the warp's smallest
-                    // and largest last state) gets the refinement's extra half interval there
-                    const int k1 = j * G0 + lane;
-                    const bool end1 = G1 == 1 && (k1 == 0 || (k1 >= gr.elo && k1 <= gr.ehi));
-                    // one-state segments away from the track ends need only the interior reach
-                    const T lim1 = G1 == 1 ? (end1 ? capth + half_rec : thin) : capth;
-                    bool hit1;
-                    if constexpr (sizeof(T) == 8)
-                        hit1 = lane < N1 &&
-                               sphere_within<float>(sph1[j * kN1Max + lane], (float)fvx, (float)fvy,
-                                                    (float)fvz, (float)fav, (float)fwx, (float)fwy,
-                                                    (float)fwz, (float)faw, (float)ax, (float)ay,
-                                                    (float)az, (float)ux, (float)uy, (float)uz,
-                                                    (float)lim1 + sph_margin_f32(fav, faw));
-                    else
-                        hit1 = lane < N1 &&
-                               sphere_within<T>(sph1[j * kN1Max + lane], fvx, fvy, fvz, fav, fwx, fwy,
-                                                fwz, faw, ax, ay, az, ux, uy, uz, lim1);
-                    const uint32_t u1 = __ballot_sync(0xffffffffu, hit1);
-                    if (u1) {
-                        // one contiguous range from the first to the last candidate level-1
-                        // segment (a superset of the candidates; their loads go out together)
-                        const int m_lo = __ffs(u1) - 1, m_hi = 31 - __clz(u1);
-                        const int sb = j * G0, se = min(sb + G0, nv);
-                        const int k0 = sb + m_lo * G1;
-                        scan(k0, min(sb + (m_hi + 1) * G1, se), (m_hi - m_lo + 1) * G1);
+                int ra = -1, rb = -1, kst = 0;
+                uint32_t near = 0xffffffffu;
+                for (bool more = true; more;) {
+                    more = false;
+                    int j = 0;
+                    uint32_t u1 = 0, key = 0;
+                    while (u0) {
+                        j = __ffs(u0) - 1;
+                        u0 &= u0 - 1;
+                        // a one-state segment that may hold a track end (the first state, or between the
+                        // warp's smallest and largest last state) gets the refinement's extra half
+                        // interval; one away from the ends needs only the interior reach
+                        const int k1 = j * G0 + lane;
+                        const bool end1 = G1 == 1 && (k1 == 0 || (k1 >= gr.elo && k1 <= gr.ehi));
+                        float d2 = 0.f;
+                        const bool hit1 = lane < N1 && sphere_within(sph1[j * kN1Max + lane], q0, q1,
+                                                                     end1 ? lim_end : lim_in, d2);
+                        u1 = __ballot_sync(0xffffffffu, hit1);
+                        if (u1) {
+                            if constexpr (F::kAxial)
+                                key = __reduce_min_sync(0xffffffffu,
+                                                        hit1 ? (__float_as_uint(d2) & ~31u) | (unsigned)lane : 0xffffffffu);
+                            more = true;
+                            break;
+                        }
+                    }
+                    const int k0 = j * G0 + (__ffs(u1) - 1) * G1;
+                    const bool joins = more && ra >= 0 && k0 <= rb + 1;
+                    if (!joins && ra >= 0) closest_in(ra, rb, kst);
+                    if (more) {
+                        if (!joins) {
+                            ra = k0;
+                            near = 0xffffffffu;
+                        }
+                        rb = min(j * G0 + (32 - __clz(u1)) * G1, min(j * G0 + G0, a.n_rec)) - 1;
+                        if ((key & ~31u) < near) {
+                            near = key & ~31u;
+                            kst = segment_centre(j * G0 + (int)(key & 31u) * G1, G1, min(j * G0 + G0, a.n_rec));
+                        }
                     }
                 }
             }
@@ -518,51 +859,46 @@ __device__ __forceinline__ void group_wires(const F &f, const DcaArgs &a, const 
             // refinement may extrapolate h_rec beyond the track); compared squared: the thresholds
             // carry margins far above the rounding of the square
             const T th = (bk == 0 || bk == nv - 1) ? capth + half_rec : thin;
-            const bool refine = want && bk != 0x7fffffff && (a.exact_all || bd <= th * th);
-            T D = T(INFINITY);
+            const bool refine = want && bk != 0x7fffffff && (ALL || !nearer<T>(th * th, bd));
+            T d = lam;   // lambda when the wire is not refined
             if (refine) {
+                T D;
                 T yv[6];
-                T s0 = T(0);
-#if COMET_DCA_SCAN_P
-#pragma unroll
-                for (int cc = 0; cc < 6; ++cc) yv[cc] = by[cc];
-                // first step to the vertex of the parabola through the squared distances of the
-                // closest state and its two neighbours (exact for a straight track, where the
-                // squared distance is quadratic in arc length); then Newton steps as usual.  Used
-                // when both neighbours were scanned and the step budget allows (max_iter >= 4).
-                if (a.max_iter >= 4 && bdm < T(INFINITY) && bdp < T(INFINITY)) {
-                    const T den = bdm - T(2) * bd + bdp;
-                    if (den > T(0)) {
-                        s0 = T(0.5) * h_rec * (bdm - bdp) / den;
-                        s0 = fmin(fmax(s0, -h_rec), h_rec);
-                    }
-                }
-#else
-                const int64_t o = (int64_t)bk * S + s;
-#pragma unroll
-                for (int cc = 0; cc < 6; ++cc) yv[cc] = P[cc * plane + o];
-#endif
-                const int conv = refine_dca<T, F>(f, gr.c, gr.ip, yv, ax, ay, az, ux, uy, uz, tol,
+                const Off o = (Off)bk * row + col;
+                yv[0] = val(0, o);
+                yv[1] = val(1, o);
+                yv[2] = val(2, o);
+                yv[3] = val(3, o);
+                yv[4] = val(4, o);
+                yv[5] = val(5, o);
+                const Q4<T> r3 = rec[4 * ii + 3];
+                const T s0 = first_step<T>(a, h_rec, bdm, bd, bdp);
+                const int conv = refine_dca<T, F>(f, gr.c, gr.ip, yv, r2.x, r2.y, r2.z, r3.x, r3.y, r3.z, tol,
                                                   a.max_iter, h_rec, D, s0);
-                if (cap >= T(0)) nunc += 1 - conv;
-                if (a.dca_out) ((T *)a.dca_out)[(int64_t)(tl.w0 + ii) * S + s] = D;
-            }
-            if (valid && cap >= T(0)) {
-                T emin = T(INFINITY);
-                if (refine) {
-                    const int hb = tl.offs[ii], he = tl.offs[ii + 1];
-                    for (int j = hb; j < he; ++j) {
-                        if (tl.msm[j]) continue;
-                        const T e = fabs(D - tl.dsm[j]);
-                        emin = e < emin ? e : emin;
-                    }
+                if (ALL) ((T *)a.dca_out)[(int64_t)(tl.w0 + ii) * S + s] = D;
+                if (used) {
+                    nunc += 1 - conv;
+                    d = residual<T>(tl, ii, D, lam, nin);
                 }
-                const T d = emin < lam ? emin : lam;
-                nin += emin < lam ? 1 : 0;
-                acc.add(d * d);
             }
+            if (used) acc.add_square(d);
         }
     }
+}
+
+// How a launch searches for the closest states.
+enum Search { kShort, kLong, kAll };   // runs of a few states; runs of many; every DCA wanted
+
+template <typename T, class F, typename Off, Search HOW>
+__device__ __forceinline__ void group_wires(const F &f, const DcaArgs &a, const Group<T> &gr,
+                                            const Tile<T> &tl, const float4 *sph0,
+                                            const float4 *sph1, int lane, Acc<T> &acc, int &nin,
+                                            int &nunc, int wb, int we)
+{
+    if constexpr (HOW == kShort)
+        group_wires_short<T, F, Off>(f, a, gr, tl, sph0, sph1, lane, acc, nin, nunc, wb, we);
+    else
+        group_wires_long<T, F, Off, HOW == kAll>(f, a, gr, tl, sph0, sph1, lane, acc, nin, nunc, wb, we);
 }
 
 // Wire chunk c of n over W wires: [c * wc, min((c + 1) * wc, W)), wc = ceil(W / n).
@@ -574,7 +910,7 @@ __device__ __forceinline__ int2 chunk_range(int W, int n, int c)
 
 // All wire chunks of one group in this warp: each chunk's partial sum, added in chunk order (the
 // arithmetic the cross-warp schedule of the persistent kernel reproduces).
-template <typename T, class F>
+template <typename T, class F, typename Off, Search HOW>
 __device__ __forceinline__ void group_all_chunks(const F &f, const DcaArgs &a, const Group<T> &gr,
                                                  const Tile<T> &tl, const float4 *sph0,
                                                  const float4 *sph1, int lane, Acc<T> &acc,
@@ -583,7 +919,7 @@ __device__ __forceinline__ void group_all_chunks(const F &f, const DcaArgs &a, c
     for (int c = 0; c < a.n_chunks; ++c) {
         const int2 r = chunk_range(tl.wn, a.n_chunks, c);
         Acc<T> part;
-        group_wires<T, F>(f, a, gr, tl, sph0, sph1, lane, part, nin, nunc, r.x, r.y);
+        group_wires<T, F, Off, HOW>(f, a, gr, tl, sph0, sph1, lane, part, nin, nunc, r.x, r.y);
         acc.add_pair(part.hi, part.lo);
     }
 }
@@ -726,11 +1062,11 @@ struct PLayout {
 // table was given; with the recording kernel's table, the part a group can use -- its kN0Max
 // super-segment spheres and the level-1 spheres of the super-segments an n_rec-state track has --
 // copied in per work item (about 1.3 KB per warp at 70 recorded states, so that the per-wire
-// level-1 tests read shared memory, not L2); none when every state is scanned (dca_out requested).
+// level-1 tests read shared memory, not L2); none when every state is scanned (dca_out requested and
+// no table given).
 __host__ __device__ inline int p_sph_entries(const DcaArgs &a)
 {
-    if (a.exact_all) return 0;
-    if (a.bounds == nullptr) return kBoundsPerGroup;
+    if (a.bounds == nullptr) return a.exact_all ? 0 : kBoundsPerGroup;
     int n0 = (a.n_rec + a.G0 - 1) / a.G0;
     n0 = n0 < kN0Max ? n0 : kN0Max;
     return kN0Max + n0 * kN1Max;
@@ -756,8 +1092,16 @@ __host__ __device__ inline PLayout p_layout(int W, int es, int nsph)
 
 constexpr int kPersistMaxW = 1024;
 
+// Resident CTAs per SM that the registers are allocated for.
 template <typename T, class F>
-__global__ void __launch_bounds__(kThreads, sizeof(T) == 8 ? COMET_DCA_MINB_F64 : (F::kAxial ? COMET_DCA_MINB : COMET_DCA_MINB_FIELD)) dca_persistent_kernel(F f, DcaArgs a)
+constexpr int min_ctas(Search how)
+{
+    return sizeof(T) == 8 ? COMET_DCA_MINB_F64
+                          : (!F::kAxial ? COMET_DCA_MINB_FIELD : (how == kLong ? COMET_DCA_MINB_LONG : COMET_DCA_MINB));
+}
+
+template <typename T, class F, typename Off, Search HOW>
+__global__ void __launch_bounds__(kThreads, min_ctas<T, F>(HOW)) dca_persistent_kernel(F f, DcaArgs a)
 {
     const bool sph_smem = a.bounds == nullptr && !a.exact_all;
     const PLayout L = p_layout(a.W, (int)sizeof(T), p_sph_entries(a));
@@ -835,8 +1179,15 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 8 ? COMET_DCA_MINB_F64 
     tl.msm = hits_sm ? msm + moff : a.mask;
     tl.w0 = 0;
     tl.wn = W;
+    tl.ff = (const float4 *)wrow;
     for (int i = tid; i < W; i += kThreads) tile_wire_setup<T>(tl, i, in_prec<T>(a.lambda, a.lambda_f), capv, frm);
     __syncthreads();
+    if constexpr (sizeof(T) == 8) {
+        // a copy given up on above may still land in the rows
+        if (any_timeout) mbar_wait(bar, parity ^ 1u, kWaitNs);
+        tile_float_frames<T>(frm, W, (float4 *)wrow);
+        __syncthreads();
+    }
 
     // ---- work items taken dynamically by each warp: 32-seed groups, or (group, wire chunk) pairs
     // when partial sums can be parked in `part` (finer items balance the warps' loads)
@@ -861,11 +1212,11 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 8 ? COMET_DCA_MINB_F64 
             for (int i = lane; i < L.nsph; i += 32) sph0[i] = __ldg(src + i);
             __syncwarp();
         }
-        const float4 *s0 = sph0, *s1 = sph1;
+        const float4 *s0 = L.nsph > 0 ? sph0 : nullptr, *s1 = sph1;
         Acc<T> acc;
         int nin = 0;
         if (!split) {
-            group_all_chunks<T, F>(f, a, gr, tl, s0, s1, lane, acc, nin, nunc);
+            group_all_chunks<T, F, Off, HOW>(f, a, gr, tl, s0, s1, lane, acc, nin, nunc);
             const T v = acc.value();
             if (gr.valid) {
                 ((T *)a.rss)[gr.s] = v;
@@ -874,7 +1225,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 8 ? COMET_DCA_MINB_F64 
             if (a.best_idx_out) group_best_fold<T>(s_best, warp, lane, gr.valid, v, gr.s);
         } else {
             const int2 r = chunk_range(W, nc, c);
-            group_wires<T, F>(f, a, gr, tl, s0, s1, lane, acc, nin, nunc, r.x, r.y);
+            group_wires<T, F, Off, HOW>(f, a, gr, tl, s0, s1, lane, acc, nin, nunc, r.x, r.y);
             T *ph = (T *)a.part;
             T *pl = ph + (size_t)nc * a.S;
             int32_t *pn = (int32_t *)(pl + (size_t)nc * a.S);
@@ -927,8 +1278,8 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 8 ? COMET_DCA_MINB_F64 
 // Tiled kernel: more wires than one tile holds.  One 128-seed block per CTA; wires staged in tiles.
 // ------------------------------------------------------------------------------------------------
 
-template <typename T, class F>
-__global__ void __launch_bounds__(kThreads, sizeof(T) == 8 ? COMET_DCA_MINB_F64 : (F::kAxial ? COMET_DCA_MINB : COMET_DCA_MINB_FIELD)) dca_tiled_kernel(F f, DcaArgs a)
+template <typename T, class F, typename Off, Search HOW>
+__global__ void __launch_bounds__(kThreads, min_ctas<T, F>(HOW)) dca_tiled_kernel(F f, DcaArgs a)
 {
     using L = Smem<T>;
     extern __shared__ __align__(128) unsigned char sm[];
@@ -949,7 +1300,8 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 8 ? COMET_DCA_MINB_F64 
     if (tid == 0) mbar_init(bar, 1);
     const int64_t g = (int64_t)blockIdx.x * kWarps + warp;
     const Group<T> gr = load_group<T>(a, g, lane);
-    if (!a.exact_all) build_spheres<T>(a, gr, lane, sph0, sph1, g);
+    const bool pruned = HOW != kAll || a.bounds;
+    if (pruned) build_spheres<T>(a, gr, lane, sph0, sph1, g);
 
     const int W = a.W;
     const int H = W > 0 ? a.offs[W] : 0;
@@ -1018,10 +1370,19 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 8 ? COMET_DCA_MINB_F64 
         tl.msm = hits_sm ? msm + moff : a.mask;
         tl.w0 = w0;
         tl.wn = wn;
+        tl.ff = (const float4 *)wrow;
         for (int i = tid; i < wn; i += kThreads) tile_wire_setup<T>(tl, i, in_prec<T>(a.lambda, a.lambda_f), capv, frm);
         __syncthreads();
-        group_wires<T, F>(f, a, gr, tl, sph0, sph1, lane, acc, nin, nunc, 0, wn);
-        if (w0 + kWireTile < W) __syncthreads();   // tile consumed before the next staging
+        if constexpr (sizeof(T) == 8) {
+            tile_float_frames<T>(frm, wn, (float4 *)wrow);
+            __syncthreads();
+        }
+        group_wires<T, F, Off, HOW>(f, a, gr, tl, pruned ? sph0 : nullptr, sph1, lane, acc, nin, nunc, 0, wn);
+        if (w0 + kWireTile < W) {
+            // tile consumed before the next staging's bulk copies overwrite it
+            fence_proxy_async_smem();
+            __syncthreads();
+        }
     }
 
     const T v = acc.value();
@@ -1057,16 +1418,16 @@ static int sm_count()
     return n;
 }
 
-template <typename T, class F>
-static cudaError_t dca_launch(const F &fld, const DcaArgs &a, cudaStream_t st)
+template <typename T, class F, typename Off, Search HOW>
+static cudaError_t dca_launch_off(const F &fld, const DcaArgs &a, cudaStream_t st)
 {
     if (a.W <= kPersistMaxW && a.counter) {
         const PLayout L = p_layout(a.W, (int)sizeof(T), p_sph_entries(a));
-        cudaError_t e = cudaFuncSetAttribute(dca_persistent_kernel<T, F>,
+        cudaError_t e = cudaFuncSetAttribute(dca_persistent_kernel<T, F, Off, HOW>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.total);
         if (e != cudaSuccess) return e;
         int per_sm = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, dca_persistent_kernel<T, F>,
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, dca_persistent_kernel<T, F, Off, HOW>,
                                                           kThreads, L.total);
         if (e != cudaSuccess) return e;
         per_sm = per_sm < 1 ? 1 : per_sm;
@@ -1078,17 +1439,37 @@ static cudaError_t dca_launch(const F &fld, const DcaArgs &a, cudaStream_t st)
         e = cudaMemsetAsync(a.counter, 0, sizeof(int32_t), st);
         if (e != cudaSuccess) return e;
         if (a.best_idx_out && nb > a.best_slots_cap) return cudaErrorInvalidValue;   // one slot per CTA
-        dca_persistent_kernel<T, F><<<(unsigned)nb, kThreads, L.total, st>>>(fld, a);
+        dca_persistent_kernel<T, F, Off, HOW><<<(unsigned)nb, kThreads, L.total, st>>>(fld, a);
         return cudaGetLastError();
     }
     using L = Smem<T>;
     static const cudaError_t attr = cudaFuncSetAttribute(
-        dca_tiled_kernel<T, F>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L::total);
+        dca_tiled_kernel<T, F, Off, HOW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L::total);
     if (attr != cudaSuccess) return attr;
     const int64_t nb = (a.S + kThreads - 1) / kThreads;
     if (a.best_idx_out && nb > a.best_slots_cap) return cudaErrorInvalidValue;   // one slot per CTA
-    dca_tiled_kernel<T, F><<<(unsigned)nb, kThreads, L::total, st>>>(fld, a);
+    dca_tiled_kernel<T, F, Off, HOW><<<(unsigned)nb, kThreads, L::total, st>>>(fld, a);
     return cudaGetLastError();
+}
+
+template <typename T, class F, Search HOW>
+static cudaError_t dca_launch_how(const F &fld, const DcaArgs &a, cudaStream_t st)
+{
+    // 32-bit offsets (one register and no carry per address) into a track array below 4 GiB
+    return 6 * a.S * (int64_t)a.n_rec * (int64_t)sizeof(T) < ((int64_t)1 << 32)
+               ? dca_launch_off<T, F, uint32_t, HOW>(fld, a, st)
+               : dca_launch_off<T, F, size_t, HOW>(fld, a, st);
+}
+
+// FP32 in an axial field takes the short form (group_wires_short) when a level-1 segment is one state:
+// runs are then a few states long.
+template <typename T, class F>
+static cudaError_t dca_launch(const F &fld, const DcaArgs &a, cudaStream_t st)
+{
+    if (a.exact_all) return dca_launch_how<T, F, kAll>(fld, a, st);
+    if constexpr (sizeof(T) == 4 && F::kAxial)
+        if (a.G1 == 1 && a.W <= kPersistMaxW) return dca_launch_how<T, F, kShort>(fld, a, st);
+    return dca_launch_how<T, F, kLong>(fld, a, st);
 }
 
 template <typename T>
@@ -1160,7 +1541,8 @@ void dca_segments(int n_rec, int *G0, int *G1)
 // ------------------------------------------------------------------------------------------------
 
 #ifndef COMET_DCA_BATCH_MINB
-#define COMET_DCA_BATCH_MINB 6   // the event's arguments come from a table, not the parameter bank
+#define COMET_DCA_BATCH_MINB 4   // the event's arguments come from a table, not the parameter bank: at 6 the
+                                 // kernel spilled (three rounds of 16 events 1438 us at 6, 1210 at 5, 1183 at 4)
 #endif
 
 template <typename T, class F>
@@ -1270,6 +1652,7 @@ __global__ void __launch_bounds__(kThreads, COMET_DCA_BATCH_MINB) dca_batch_kern
                 s_tl.uy = wrow + 4 * rcap + woff[4];
                 s_tl.uz = wrow + 5 * rcap + woff[5];
                 s_tl.rec = frm;
+                s_tl.ff = (const float4 *)wrow;
                 s_tl.cap = capv;
                 s_tl.offs = orow + ooff;
                 s_tl.dsm = hits_sm ? dsm + doff : Dg;
@@ -1280,6 +1663,10 @@ __global__ void __launch_bounds__(kThreads, COMET_DCA_BATCH_MINB) dca_batch_kern
             __syncthreads();
             for (int i = tid; i < W; i += kThreads) tile_wire_setup<T>(tl, i, in_prec<T>(a.lambda, a.lambda_f), capv, frm);
             __syncthreads();
+            if constexpr (sizeof(T) == 8) {
+                tile_float_frames<T>(frm, W, (float4 *)wrow);
+                __syncthreads();
+            }
         }
         // the item's (group, wire chunk) sub-items, taken by the warps as they come free
         const int nc = a.n_chunks;
@@ -1303,7 +1690,7 @@ __global__ void __launch_bounds__(kThreads, COMET_DCA_BATCH_MINB) dca_batch_kern
             Acc<T> acc;
             int nin = 0;
             const int2 r = chunk_range(a.W, nc, k % nc);
-            group_wires<T, F>(f, a, gr, tl, s0, s0 + kN0Max, lane, acc, nin, nunc, r.x, r.y);
+            group_wires<T, F, size_t, kShort>(f, a, gr, tl, s0, s0 + kN0Max, lane, acc, nin, nunc, r.x, r.y);
             ph[k * 32 + lane] = acc.hi;
             pl[k * 32 + lane] = acc.lo;
             pn[k * 32 + lane] = nin;

@@ -125,6 +125,41 @@ def test_jacobian_lane_groups(ctx, n_seeds, n_wires, stride):
 
 
 @pytest.mark.parametrize("dtype", [torch.float32, torch.float64])
+@pytest.mark.parametrize("stride,n_seeds,zmax", [(1, 64, 9.0), (2, 33, 9.0), (8, 97, 9.0), (11, 64, 9.0), (12, 40, 9.0),
+                                                 (16, 1, 9.0), (32, 64, 9.0), (32, 97, -0.3), (1, 40, -0.3)])
+def test_closest_state_without_scanning_equals_the_scan(ctx, dtype, stride, n_seeds, zmax):
+    """The walk down a track's valley and the spheres' bounds against the scan of every recorded state
+    (DCAs wanted, no spheres given): the same DCAs, sums and counts, bit for bit.  Level-1 segments of one
+    state (more than 192 states have several each), runs across super-segments, tracks that leave the
+    region, chamber wires, wires of any direction (along the tracks too, where the valley is not
+    convex and is scanned) and wires around the helix axis, which every state is equally far from."""
+    ev = synth.multi_turn_event(1, counts=(8, 8, 16, 8))
+    spec = ev.partitions[0]
+    seeds = O.lattice(spec)[:n_seeds]
+    rng = np.random.default_rng(stride)
+    path, _ = O.propagate(UNIFORM, O.Params(n_steps=ev.n_steps[0], stride=1), seeds[:1], spec.charge)
+    n = 60
+    at = path[0, rng.integers(0, path.shape[1], n), :3] + rng.normal(scale=6e-3, size=(n, 3))
+    u = rng.normal(size=(n, 3)) * [1.0, 1.0, 2.0]
+    u /= np.linalg.norm(u, axis=1, keepdims=True)
+    centre = path[0, :, :3].mean(0)
+    wires = np.concatenate([ev.wires, np.concatenate([at, u], 1).T,
+                            np.array([[*centre, 0.0, 0.0, 1.0], [*path[0, 0, :3], 0.0, 0.0, 1.0]]).T], axis=1)
+    W = wires.shape[1]
+    offs = np.arange(W + 1, dtype=np.int32)
+    drift = rng.uniform(0.0, 8e-3, W)
+    mask = (rng.random(W) < 0.1).astype(np.uint8)
+    bp = B.ScanParams(n_steps=ev.n_steps[0], stride=stride, zmax=zmax, lam=1e-2)
+
+    def run(p, want_dca, use_bounds):
+        return gpu_dca(ctx, B.DeviceField.from_synth(UNIFORM), p, seeds, spec.charge, wires, offs, drift, mask, dtype,
+                       want_dca=want_dca, use_bounds=use_bounds)
+    full, kept = run(bp, True, False), run(bp, True, True)
+    for name in ("dca", "rss", "n_in"):
+        assert np.array_equal(full[name], kept[name])
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.float64])
 @pytest.mark.parametrize("k,counts,want_dca", [(1, (2, 3, 4, 5), False), (1, (1, 1, 1, 1), True), (10, (3, 4, 5, 6), True),
                                                (64, (4, 4, 4, 4), False)])
 def test_partition_in_one_call_equals_the_five(ctx, dtype, k, counts, want_dca):
