@@ -73,6 +73,7 @@ struct FieldTable {
     int nx, ny, nz;
     T ox, oy, oz, inv_sp;
     int il;   // layout: 0 = [3][nz][ny][nx], 1 = [nz][ny][nx][4] (one 16-byte load per node)
+    int mx, my, mz;   // cells a side for cell_fast (0: the grid is too long for it)
 
     __device__ __forceinline__ static void cell(T g, int n, int &i, T &t)
     {
@@ -82,6 +83,21 @@ struct FieldTable {
         i = (int)fl;
         i = i > n - 2 ? n - 2 : i;
         t = g - T(i);
+    }
+
+    // The same for a float g inside a grid of m < 2^22 cells a side (false where it is not inside, or not
+    // a number): the floor and its integer by adding 1.5 2^23, whose ulp is 1, rounded down, in place
+    // of the conversions (a quarter of the float rate here); no clamping is needed inside.  Recording in
+    // the tabulated field, 2^18 seeds x 2,204 steps: 7778 -> 7659 us (with the in-cell test as integers).
+    // Not for single lookups (at): the DCA's refinement there went from 655 to 707 us, spilling.
+    __device__ __forceinline__ static bool cell_fast(float g, int m, int &i, T &fi, T &t)
+    {
+        constexpr float kOne = 12582912.f;
+        const float r = __fadd_rd(g, kOne);
+        i = __float_as_int(r) - 0x4b400000;
+        fi = __fsub_rn(r, kOne);
+        t = __fsub_rn(g, (float)fi);
+        return (unsigned)i < (unsigned)m;
     }
 
     // The eight corner nodes of the grid cell a lane used last (base: index of its node 000; none
@@ -114,8 +130,12 @@ struct FieldTable {
         // inside the cached cell, 0 <= g - i < 1 in every dimension: g needs no clamping there,
         // floor(g) = i, and g - i is exact (Sterbenz), so these are the fractions cell() gives
         T tx = gx - cc.fx, ty = gy - cc.fy, tz = gz - cc.fz;
-        if (!(tx >= T(0) && tx < T(1) && ty >= T(0) && ty < T(1) && tz >= T(0) && tz < T(1)))
-            enter(cc, gx, gy, gz, tx, ty, tz);
+        bool same;
+        if constexpr (sizeof(T) == 4)   // as integers: negative values and NaN are above 1
+            same = max(max(__float_as_uint(tx), __float_as_uint(ty)), __float_as_uint(tz)) < 0x3f800000u;
+        else
+            same = tx >= T(0) && tx < T(1) && ty >= T(0) && ty < T(1) && tz >= T(0) && tz < T(1);
+        if (!same) enter(cc, gx, gy, gz, tx, ty, tz);
         bx = lerp3(cc, 0, tx, ty, tz);
         by = lerp3(cc, 1, tx, ty, tz);
         bz = lerp3(cc, 2, tx, ty, tz);
@@ -136,12 +156,20 @@ struct FieldTable {
     __device__ __forceinline__ void enter(Cell &cc, T gx, T gy, T gz, T &tx, T &ty, T &tz) const
     {
         int ix, iy, iz;
-        cell(gx, nx, ix, tx);
-        cell(gy, ny, iy, ty);
-        cell(gz, nz, iz, tz);
-        cc.fx = T(ix);
-        cc.fy = T(iy);
-        cc.fz = T(iz);
+        bool in = false;
+        if constexpr (sizeof(T) == 4) {
+            const bool jx = cell_fast(gx, mx, ix, cc.fx, tx), jy = cell_fast(gy, my, iy, cc.fy, ty),
+                       jz = cell_fast(gz, mz, iz, cc.fz, tz);
+            in = jx && jy && jz;
+        }
+        if (!in) {
+            cell(gx, nx, ix, tx);
+            cell(gy, ny, iy, ty);
+            cell(gz, nz, iz, tz);
+            cc.fx = T(ix);
+            cc.fy = T(iy);
+            cc.fz = T(iz);
+        }
         const int64_t base = ((int64_t)iz * ny + iy) * nx + ix;
         if (base != cc.base) {
             cc.base = base;
@@ -231,7 +259,9 @@ template <typename T>
 inline FieldTable<T> make_table(const comet_field &f)
 {
     return FieldTable<T>{(const float *)f.table, f.nx, f.ny, f.nz, (T)f.origin[0], (T)f.origin[1],
-                         (T)f.origin[2], (T)(1.0 / f.spacing), f.kind == 2 ? 1 : 0};
+                         (T)f.origin[2], (T)(1.0 / f.spacing), f.kind == 2 ? 1 : 0,
+                         f.nx <= (1 << 22) ? f.nx - 1 : 0, f.ny <= (1 << 22) ? f.ny - 1 : 0,
+                         f.nz <= (1 << 22) ? f.nz - 1 : 0};
 }
 
 // ------------------------------------------------------------------------------------------------

@@ -186,3 +186,24 @@ def test_partition_in_one_call_equals_the_five(ctx, dtype, k, counts, want_dca):
     small = scan.Workspace(max(spec.n_seeds - 1, 1), bp.n_rec - 1, ev.n_hits, dtype, k=k)
     with pytest.raises(RuntimeError):
         scan.scan_partition(ctx, B.DeviceField.from_synth(UNIFORM), bp, spec, dev, small, k=k)
+
+
+@pytest.mark.parametrize("interleaved", [False, True])
+@pytest.mark.parametrize("half,n", [(0.9, 37), (0.25, 11), (0.0625, 2), (0.5, 3)])
+def test_fp32_field_cells_and_the_grid_edge(ctx, half, n, interleaved):
+    """FP32 recording in a table that the track leaves, enters and runs along (seeds on nodes, on the edge
+    and outside, where coordinates are clamped; a grid of one cell) against the FP64 kernel, whose cells
+    come from the general lookup: within 1 um, the bar of the FP32 points."""
+    g = np.linspace(-half, half, n)
+    z, y, x = np.meshgrid(g, g, g, indexing="ij")
+    table = np.stack([0.03 * z + 0.02 * y, 0.05 * x * z, 1.0 + 0.1 * x - 0.05 * y * z]).astype(np.float32)
+    field = B.DeviceField(1, table=table, origin=(-half,) * 3, spacing=2 * half / (n - 1), interleaved=interleaved)
+    start = [(0.0, 0.0, 0.0), (half, 0.0, 0.0), (-half, half, -half), (0.0, -half, half), (half + 0.01, 0.02, 0.0),
+             (g[n // 2], g[0], g[n // 2]), (-0.05, 0.04, -half - 0.02)]
+    seeds = np.array([[*p, 90.0 * np.cos(a), 90.0 * np.sin(a), 20.0] for p in start for a in (0.0, 1.3, 2.9, 4.4, 5.6)])
+    bp = B.ScanParams(n_steps=1600, stride=8, zmin=-9.0, zmax=9.0, rmax=9.0)
+    seeds = seeds.astype(np.float32).astype(np.float64)
+    _, _, p32, n32 = gpu_propagate(ctx, field, bp, seeds, -1, torch.float32)
+    _, _, p64, n64 = gpu_propagate(ctx, field, bp, seeds, -1, torch.float64)
+    assert torch.equal(n32, n64)
+    assert float((p32[:3].double() - p64[:3]).abs().max()) < 1e-6
