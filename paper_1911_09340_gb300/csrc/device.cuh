@@ -675,11 +675,12 @@ constexpr int kBoundsPerGroup = kN0Max + kN0Max * kN1Max;
 // Centre index of a lane's segment [st, st + g) inside [.., end) (end = its last state + 1).
 __device__ __forceinline__ int segment_centre(int st, int g, int end) { return min(st + g / 2, min(st + g, end) - 1); }
 
-// A group's spread about a segment's centre states: the midpoint of two of its lanes' centres, the
-// square m2 of the largest distance from it to any lane's centre, and rs about 1 / sqrt(m2).
+// A group's spread about a segment's centre states: the sum of two of its lanes' centres (twice their
+// midpoint), the square m2 of the largest distance from the midpoint to any lane's centre, and rs
+// about 1 / sqrt(m2).
 template <typename T>
 struct WarpSpread {
-    T cx, cy, cz;
+    T sx, sy, sz;
     float m2, rs;
 };
 
@@ -690,18 +691,20 @@ template <typename T>
 __device__ __forceinline__ WarpSpread<T> warp_spread(bool has, int l0, int l1, T x, T y, T z)
 {
     WarpSpread<T> w;
-    w.cx = T(0.5) * (__shfl_sync(0xffffffffu, x, l0) + __shfl_sync(0xffffffffu, x, l1));
-    w.cy = T(0.5) * (__shfl_sync(0xffffffffu, y, l0) + __shfl_sync(0xffffffffu, y, l1));
-    w.cz = T(0.5) * (__shfl_sync(0xffffffffu, z, l0) + __shfl_sync(0xffffffffu, z, l1));
+    w.sx = __shfl_sync(0xffffffffu, x, l0) + __shfl_sync(0xffffffffu, x, l1);
+    w.sy = __shfl_sync(0xffffffffu, y, l0) + __shfl_sync(0xffffffffu, y, l1);
+    w.sz = __shfl_sync(0xffffffffu, z, l0) + __shfl_sync(0xffffffffu, z, l1);
+    // half of a sum is exact, so these round once, as x - midpoint does
+    const T dx = fma(T(-0.5), w.sx, x), dy = fma(T(-0.5), w.sy, y), dz = fma(T(-0.5), w.sz, z);
     // d^2 >= 0 as a float (rounded up from double): its bit pattern orders like its value, so one
     // integer warp reduction finds the max; then one root by the hardware reciprocal square root
     // (a few ulp, inside the 1e-6 relative margin of the radius).  The radius is a float either way,
     // so the double path needs no double root or reductions (this part's FP64 rate is small).
     float d2;
     if constexpr (sizeof(T) == 4)
-        d2 = has ? (x - w.cx) * (x - w.cx) + (y - w.cy) * (y - w.cy) + (z - w.cz) * (z - w.cz) : 0.f;
+        d2 = has ? dx * dx + dy * dy + dz * dz : 0.f;
     else
-        d2 = has ? __double2float_ru((x - w.cx) * (x - w.cx) + (y - w.cy) * (y - w.cy) + (z - w.cz) * (z - w.cz)) : 0.f;
+        d2 = has ? __double2float_ru(dx * dx + dy * dy + dz * dz) : 0.f;
     w.m2 = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(d2)));
     w.rs = rsqrtf(fmaxf(w.m2, 1e-30f));
     return w;
@@ -719,7 +722,7 @@ __device__ __forceinline__ float4 spread_sphere(const WarpSpread<T> &w, T reach)
         rad = __fmul_rn(__fmaf_rn(w.m2, w.rs, reach), 1.000001f);
     else
         rad = (float)(((T)(w.m2 * w.rs) + reach + T(2e-7)) * T(1.000001));
-    return make_float4((float)w.cx, (float)w.cy, (float)w.cz, rad);
+    return make_float4((float)(T(0.5) * w.sx), (float)(T(0.5) * w.sy), (float)(T(0.5) * w.sz), rad);
 }
 
 // The warp's bounding sphere of one segment; radius < 0 when no lane has the segment.

@@ -335,12 +335,23 @@ __device__ __forceinline__ void record_inside(const F &f, const PropArgs &a, con
     float4 *t1 = tab + kN0Max;   // next level-1 entry
     int m = 0;
     if (G1 == 1) {
+        // FP64: forming a sphere from its spread takes 11 FP64 instructions, so 32 states' spreads are kept,
+        // one per lane, and their spheres formed together (2^15 seeds x 139 states, with the midpoints
+        // left as sums: 349 -> 246 us)
+        WarpSpread<T> kept{};
         auto emit = [&](const WarpSpread<T> &w, int k) {
-            if (lane == 0) *t1 = spread_sphere<T>(w, R1);
-            ++t1;
-            if (++m == G0) {
-                m = 0;
-                t1 += kN1Max - G0;
+            if constexpr (sizeof(T) == 8) {
+                if (lane == (k & 31)) kept = w;
+                const int mine = (k & ~31) + lane;
+                if (((k & 31) == 31 || k == n_rec - 1) && mine <= k)
+                    t1[mine / G0 * kN1Max + mine % G0] = spread_sphere<T>(kept, R1);
+            } else {
+                if (lane == 0) *t1 = spread_sphere<T>(w, R1);
+                ++t1;
+                if (++m == G0) {
+                    m = 0;
+                    t1 += kN1Max - G0;
+                }
             }
             if (k == c0) super(w);
         };
