@@ -623,14 +623,23 @@ __device__ __forceinline__ int refine_dca(const F &f, T c, T ip, T y[6], T ax, T
         const T tu = tx * ux + ty * uy + tz * uz;
         const T nx = tx - tu * ux, ny = ty - tu * uy, nz = tz - tu * uz;
         const T nn2 = nx * nx + ny * ny + nz * nz;
-        if (nn2 < T(1e-18)) break;
+        // FP64 leaves as soon as it can (each instruction holds its scheduler for 64 cycles); FP32 has one
+        // exit for all reasons, below: four branches an iteration were a tenth of its instructions (DCA of
+        // 2^18 seeds x 70 states 449 -> 425 us)
+        const bool flat = nn2 < T(1e-18);
+        if (sizeof(T) == 8 && flat) break;
         const T rn = rsqrt_t<T>(nn2);
         const T dist = ((y[0] - ax) * nx + (y[1] - ay) * ny + (y[2] - az) * nz) * rn;
-        if (fabs(dist) < tol) {
-            conv = 1;
-            break;
+        const bool there = fabs(dist) < tol;
+        if constexpr (sizeof(T) == 8) {
+            if (there) {
+                conv = 1;
+                break;
+            }
+            if (it >= max_iter) break;
+        } else {
+            conv = there && !flat;
         }
-        if (it >= max_iter) break;
         T step = dist * rn;
         if constexpr (F::kAxial && sizeof(T) == 8) {
             // |n| ds is not all of the plane distance's change: the plane turns by curv ds too, so each step
@@ -648,10 +657,14 @@ __device__ __forceinline__ int refine_dca(const F &f, T c, T ip, T y[6], T ax, T
             step *= (T)gain;
         }
         T target = sigma - step;
-        target = target > h_rec ? h_rec : target;
-        target = target < -h_rec ? -h_rec : target;
+        if constexpr (sizeof(T) == 8) {
+            target = target > h_rec ? h_rec : target;
+            target = target < -h_rec ? -h_rec : target;
+        } else {
+            target = fmaxf(fminf(target, h_rec), -h_rec);
+        }
         const T ds = target - sigma;
-        if (ds == T(0)) break;
+        if (ds == T(0) || (sizeof(T) == 4 && (flat || conv || it >= max_iter))) break;
         rk4_step<T, F>(f, c, ip, y, ds);
         sigma = target;
     }
