@@ -825,8 +825,14 @@ __device__ __forceinline__ void group_wires_long(const F &f, const DcaArgs &a, c
                         const int k1 = j * G0 + lane;
                         const bool end1 = G1 == 1 && (k1 == 0 || (k1 >= gr.elo && k1 <= gr.ehi));
                         float d2 = 0.f;
-                        const bool hit1 = lane < N1 && sphere_within(sph1[j * kN1Max + lane], q0, q1,
-                                                                     end1 ? lim_end : lim_in, d2);
+                        bool hit1 = false;
+                        if (lane < N1) {
+                            const float4 sp = sph1[j * kN1Max + lane];
+                            hit1 = sphere_within(sp, q0, q1, end1 ? lim_end : lim_in, d2);
+                            // every DCA wanted: a sphere that a track which is not finite has spoilt
+                            // excludes nothing
+                            if (ALL) hit1 |= !(sp.w * d2 < INFINITY);
+                        }
                         u1 = __ballot_sync(0xffffffffu, hit1);
                         if (u1) {
                             if constexpr (F::kAxial)

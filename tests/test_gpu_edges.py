@@ -160,6 +160,26 @@ def test_closest_state_without_scanning_equals_the_scan(ctx, dtype, stride, n_se
 
 
 @pytest.mark.parametrize("dtype", [torch.float32, torch.float64])
+@pytest.mark.parametrize("stride,bad", [(1, 0), (16, 5), (16, 31), (32, 33)])
+@pytest.mark.parametrize("value", [float("nan"), float("inf")])
+def test_every_dca_beside_a_track_that_is_not_finite(ctx, dtype, stride, bad, value):
+    """A seed that is not finite spoils its group's spheres; when every DCA is wanted the other seeds of
+    the group still get theirs, as without spheres."""
+    ev = synth.multi_turn_event(1, counts=(4, 4, 4, 2))
+    spec = ev.partitions[0]
+    seeds = O.lattice(spec)[:70].copy()
+    seeds[bad, 3] = value
+    W = ev.n_wires
+    bp = B.ScanParams(n_steps=ev.n_steps[0], stride=stride, lam=1e-2)
+    full, kept = (gpu_dca(ctx, B.DeviceField.from_synth(UNIFORM), bp, seeds, spec.charge, ev.wires, ev.hit_offsets,
+                          ev.drift, np.zeros(ev.n_hits, np.uint8), dtype, want_dca=True, use_bounds=b) for b in (False, True))
+    others = np.arange(70) != bad
+    assert full["dca"].shape == (70, W) and np.isfinite(full["dca"][others]).all()
+    for name in ("dca", "rss", "n_in"):
+        assert np.array_equal(full[name], kept[name], equal_nan=True)
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.float64])
 @pytest.mark.parametrize("k,counts,want_dca", [(1, (2, 3, 4, 5), False), (1, (1, 1, 1, 1), True), (10, (3, 4, 5, 6), True),
                                                (64, (4, 4, 4, 4), False)])
 def test_partition_in_one_call_equals_the_five(ctx, dtype, k, counts, want_dca):
