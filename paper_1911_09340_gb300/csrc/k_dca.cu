@@ -372,6 +372,22 @@ __device__ __forceinline__ T interior_margin(const F &f, const DcaArgs &a, const
     return T(0.5) * warp_curvature<T, F>(f, gr) * half_rec * half_rec + in_prec<T>(a.margin, a.margin_f);
 }
 
+// Lane m's one-state segments m that may hold a track end, a bit per super-segment: the first state, or
+// between the warp's smallest and largest last state.  The others need only the interior reach.  (Formed
+// once per item in the long form: tabulated field 638 -> 612 us; in the short form the registers it costs made
+// 76,545 x 139 states 512 -> 530 us.)
+template <typename T>
+__device__ __forceinline__ uint32_t end_segments(const DcaArgs &a, const Group<T> &gr, int lane)
+{
+    uint32_t ends = 0;
+    if (a.G1 == 1)
+        for (int j = 0; j < gr.n0w; ++j) {
+            const int k = j * a.G0 + lane;
+            if (k == 0 || (k >= gr.elo && k <= gr.ehi)) ends |= 1u << j;
+        }
+    return ends;
+}
+
 // First refinement step, to the vertex of the parabola through the squared distances of the
 // closest state and its two neighbours (exact for a straight track, where the squared distance is
 // quadratic in arc length); then Newton steps as usual.  0 (none) unless both neighbours were
@@ -627,6 +643,7 @@ __device__ __forceinline__ void group_wires_long(const F &f, const DcaArgs &a, c
     const Q4<T> *rec = tl.rec;
     constexpr int kU = COMET_DCA_U2;
     const T kq2 = interior_margin<T, F>(f, a, gr);
+    const uint32_t ends = end_segments<T>(a, gr, lane);
     // for the walk to the closest state (see below)
     [[maybe_unused]] float szw = 0.f, dcv_k = 0.f, hg_k = 0.f;
     if constexpr (F::kAxial) {
@@ -819,16 +836,12 @@ __device__ __forceinline__ void group_wires_long(const F &f, const DcaArgs &a, c
                     while (u0) {
                         j = __ffs(u0) - 1;
                         u0 &= u0 - 1;
-                        // a one-state segment that may hold a track end (the first state, or between the
-                        // warp's smallest and largest last state) gets the refinement's extra half
-                        // interval; one away from the ends needs only the interior reach
-                        const int k1 = j * G0 + lane;
-                        const bool end1 = G1 == 1 && (k1 == 0 || (k1 >= gr.elo && k1 <= gr.ehi));
+                        // a segment that may hold a track end gets the refinement's extra half interval
                         float d2 = 0.f;
                         bool hit1 = false;
                         if (lane < N1) {
                             const float4 sp = sph1[j * kN1Max + lane];
-                            hit1 = sphere_within(sp, q0, q1, end1 ? lim_end : lim_in, d2);
+                            hit1 = sphere_within(sp, q0, q1, ends >> j & 1u ? lim_end : lim_in, d2);
                             // every DCA wanted: a sphere that a track which is not finite has spoilt
                             // excludes nothing
                             if (ALL) hit1 |= !(sp.w * d2 < INFINITY);
