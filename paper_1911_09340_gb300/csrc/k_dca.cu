@@ -460,10 +460,12 @@ constexpr int kWalkMin = sizeof(T) == 4 ? 10 : 4;
 // with its momentum loaded beside its position, so that the refinement starts without another round trip
 // to memory (with few warps resident, latency counts as much as issue).  Otherwise group_wires_long:
 // positions only, runs of many states walked, and the search bounded by the spheres when every DCA
-// is wanted.  Both are bound by instruction issue (72% of it used at 2^18 seeds), the refinement taking
-// the larger part.  Before (one form, 64-bit addresses, momentum selected along) and after, FP32: 2^18 seeds
-// x 70 states 463 -> 449 us, 76,545 x 139 592 -> 514, 2^14 x 2,229 560 -> 157, every DCA of 2^14 x 70
-// 373 -> 101; FP64: 4,096 x 2,229 808 -> 280, 2^15 x 139 1415 -> 1250.
+// is wanted.  The short form is bound by instruction issue (72% of it used at 2^18 seeds), the refinement
+// taking about half; the long one by the latency of the walk's loads in FP32, by the FP64 pipe in FP64.
+// Before (one form, 64-bit addresses, momentum selected along) and now, FP32: 2^18 seeds x 70 states
+// 463 -> 425 us (449 before refine_dca's single exit), 76,545 x 139 592 -> 510, 2^14 x 2,229 560 -> 156, every
+// DCA of 2^14 x 70 373 -> 102; FP64: 4,096 x 2,229 808 -> 245, 2^15 x 139 1415 -> 963 (280 and 1210
+// before refine_dca's shorter iteration and the comparisons off the FP64 pipe).
 // Off: the byte offset of a recorded value, 32 bits when the track array is small enough.
 template <typename T, class F, typename Off>
 __device__ __forceinline__ void group_wires_short(const F &f, const DcaArgs &a, const Group<T> &gr,
