@@ -198,8 +198,8 @@ comet_status comet_scan_propagate(comet_ctx *ctx, comet_dtype dtype, const comet
 
 /* ---- a4-a6: DCA finding and RSS (Algorithm 2, Eq. 1, Sec. 2.2.2) --------------------------------
  *   points, n_valid, charge, S   as written by comet_scan_propagate with the same params.
- *   bounds       optional (NULL: built here), the bounds comet_scan_propagate wrote for these
- *                points with the same params.
+ *   bounds       optional (NULL: built here, or with dca_out every state scanned), the bounds
+ *                comet_scan_propagate wrote for these points with the same params.
  *   wires        SoA [6][ldw] T: (a_x, a_y, a_z, u_x, u_y, u_z) of wire i in column i: a point on
  *                the wire and its unit direction.  ldw >= W is the row stride in elements.
  *   W            number of wires (>= 0).  W = 0 gives rss = 0 and n_in = 0.
