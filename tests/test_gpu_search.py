@@ -1,0 +1,58 @@
+"""The closest-state search and the refinement where they can go wrong: tracks that are not finite or too far
+away to square, runs of candidate states that a track's valley leaves, and the refinement's precision."""
+import numpy as np
+import pytest
+import torch
+
+from paper_1911_09340_gb300 import binding as B
+from paper_1911_09340_gb300 import synth
+
+from gpu_util import gpu_dca
+
+pytestmark = pytest.mark.gpu
+KAPPA = 299.792458
+
+
+def test_fp64_refinement_step_is_full_precision(ctx):
+    """One Newton step of up to half a metre from the recorded state (max_iter = 1, RK4 step 1 m), against
+    the same step in extended precision from the device's own states.  The step is not stationary in its
+    length there, so a relative error of the reciprocal root shows in the DCA with up to half its size in
+    metres.  Coordinates stay below 8 m and some thirty roundings of 2^-53 reach the result: 32 x 8 x 1.1e-16."""
+    rng = np.random.default_rng(5)
+    S, n = 64, 60
+    mom = rng.normal(size=(S, 3)) * [60.0, 60.0, 30.0] + [40.0, 0.0, 0.0]
+    seeds = np.concatenate([rng.uniform(-0.2, 0.2, (S, 3)), mom], axis=1)
+    u = rng.normal(size=(n, 3))
+    u /= np.linalg.norm(u, axis=1, keepdims=True)
+    wires = np.concatenate([rng.uniform(-1.5, 1.5, (n, 3)), u], axis=1).T
+    bz = 0.05
+    bp = B.ScanParams(h=1.0, n_steps=3, stride=1, zmin=-90.0, zmax=90.0, rmax=90.0, tol=1e-12, max_iter=1)
+    out = gpu_dca(ctx, B.DeviceField.from_synth(synth.uniform_field(bz)), bp, seeds, -1, wires, np.arange(n + 1),
+                  np.full(n, 1e-3), np.zeros(n, np.uint8), torch.float64, use_bounds=False)
+    L = np.longdouble
+    P = out["pts"].cpu().numpy().astype(L)                       # [6][n_rec][S]
+    A, U = wires[:3].astype(L), wires[3:].astype(L)
+    d = P[:3, :, :, None] - A[:, None, None, :]
+    e = d - (d * U[:, None, None, :]).sum(0) * U[:, None, None, :]
+    d2 = (e * e).sum(0)                                          # [n_rec][S][n]
+    k = d2.argmin(0)
+    two = np.sort(d2, axis=0)
+    clear = two[1] - two[0] > 1e-9
+    y = np.take_along_axis(P[:, :, :, None], k[None, None], axis=1)[:, 0]   # [6][S][n]
+    p0 = np.sqrt((P[3:, 0] ** 2).sum(0))[:, None]
+    t = y[3:] / p0
+    nv = t - (t * U[:, None, :]).sum(0) * U[:, None, :]
+    nn = np.sqrt((nv * nv).sum(0))
+    ds = np.clip(-((y[:3] - A[:, None, :]) * nv).sum(0) / nn / nn, -1, 1)
+    # one RK4 step of length ds in a uniform axial field: P' = m P, X' = X + N P
+    th, hp = ds * (L(KAPPA) * -1 * L(bz) / p0), ds / p0
+    m = 1 - th * th * (L(1) / 2 - th * th / 24) - 1j * (th * (1 - th * th / 6))
+    N = hp * (1 - th * th / 6) - 1j * (hp * th * (L(1) / 2 - th * th / 24))
+    X = y[0] + 1j * y[1] + N * (y[3] + 1j * y[4])
+    assert m.dtype == np.clongdouble
+    r = np.stack([X.real, X.imag, y[2] + ds * y[5] / p0]) - A[:, None, :]
+    er = r - (r * U[:, None, :]).sum(0) * U[:, None, :]
+    D = np.sqrt((er * er).sum(0))
+    usable = clear & (np.abs(ds) < 0.999) & (nn > 0.1)
+    assert usable.mean() > 0.3 and np.abs(ds)[usable].max() > 0.4
+    assert np.abs(out["dca"] - D.astype(np.float64))[usable].max() <= 32 * 8 * 2.0 ** -53
