@@ -844,9 +844,6 @@ __device__ __forceinline__ void group_wires_long(const F &f, const DcaArgs &a, c
                         if (lane < N1) {
                             const float4 sp = sph1[j * kN1Max + lane];
                             hit1 = sphere_within(sp, q0, q1, ends >> j & 1u ? lim_end : lim_in, d2);
-                            // every DCA wanted: a sphere that a track which is not finite has spoilt
-                            // excludes nothing
-                            if (ALL) hit1 |= !(sp.w * d2 < INFINITY);
                         }
                         u1 = __ballot_sync(0xffffffffu, hit1);
                         if (u1) {

@@ -4,12 +4,14 @@ import numpy as np
 import pytest
 import torch
 
+import oracle as O
 from paper_1911_09340_gb300 import binding as B
-from paper_1911_09340_gb300 import synth
+from paper_1911_09340_gb300 import scan, synth
 
-from gpu_util import gpu_dca
+from gpu_util import FP32_DCA_TOL, gpu_dca, per_wire_residual, rss_bound, seen
 
 pytestmark = pytest.mark.gpu
+UNIFORM = synth.uniform_field(1.0)
 KAPPA = 299.792458
 
 
@@ -56,3 +58,28 @@ def test_fp64_refinement_step_is_full_precision(ctx):
     usable = clear & (np.abs(ds) < 0.999) & (nn > 0.1)
     assert usable.mean() > 0.3 and np.abs(ds)[usable].max() > 0.4
     assert np.abs(out["dca"] - D.astype(np.float64))[usable].max() <= 32 * 8 * 2.0 ** -53
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.float64])
+@pytest.mark.parametrize("use_bounds", [False, True])
+@pytest.mark.parametrize("stride,bad", [(1, 0), (4, 33), (16, 5), (32, 31)])
+@pytest.mark.parametrize("value", [float("nan"), float("inf"), 0.0])
+def test_sums_beside_a_track_that_is_not_finite(ctx, dtype, use_bounds, stride, bad, value):
+    """A seed that is not finite (or has no momentum, so that its states are not) leaves the sums of the other
+    seeds of its group as they are: against the oracle's, within the DCA bars' bound."""
+    ev = synth.multi_turn_event(1, counts=(4, 4, 4, 2))
+    spec = ev.partitions[0]
+    seeds = seen(O.lattice(spec)[:70], dtype).copy()
+    others = np.arange(70) != bad
+    drift, wires, lam = seen(ev.drift, dtype), seen(ev.wires, dtype), 1e-2
+    mask = np.zeros(ev.n_hits, np.uint8)
+    op, bp = (c(n_steps=ev.n_steps[0], stride=stride, lam=lam) for c in (O.Params, B.ScanParams))
+    ref = O.scan(UNIFORM, op, seeds[others], spec.charge, O.wires_aos(wires), ev.hit_offsets, drift, mask, want_dca=True)
+    seeds[bad, 3:] = value
+    got = gpu_dca(ctx, B.DeviceField.from_synth(UNIFORM), bp, seeds, spec.charge, wires, ev.hit_offsets, drift, mask, dtype,
+                  want_dca=False, use_bounds=use_bounds)
+    delta = FP32_DCA_TOL if dtype == torch.float32 else 1e-9
+    e = per_wire_residual(ref["dca"], ev.hit_offsets, drift, mask)
+    assert (np.abs(got["rss"][others] - ref["rss"]) <= rss_bound(e, lam, delta, dtype == torch.float32) + 1e-15).all()
+    edge = (np.abs(e - lam) <= delta).sum(1)
+    assert (np.abs(got["n_in"][others] - ref["n_in"]) <= edge).all() and (ref["n_in"] > 0).any()
