@@ -216,7 +216,8 @@ comet_status comet_scan_propagate(comet_ctx *ctx, comet_dtype dtype, const comet
  *                most 32 wires (FP32 as a compensated TwoSum pair, FP64 plainly), the chunk sums
  *                then in chunk order: deterministic, independent of the GPU's scheduling.
  *   n_in         out, [S] int32: wires whose capped residual is below lambda.
- *   dca_out      optional out, [W][S] T (NULL to skip): D_i of every (wire, seed).  Requesting it
+ *   dca_out      optional out, [W][S] T (NULL to skip): D_i of every (wire, seed), NaN where no
+ *                recorded state has a distance (a track that is not finite).  Requesting it
  *                computes the exact DCA of every wire; without it, a wire the track never comes
  *                within (max drift + lambda + half a recording interval; a whole interval at the
  *                first and the last recorded state, which the refinement can move beyond) of is

@@ -871,6 +871,13 @@ __device__ __forceinline__ void group_wires_long(const F &f, const DcaArgs &a, c
                 }
             }
 
+            if constexpr (ALL) {
+                // no squared distance is below infinity: the first that overflows, if there is one
+                if (want && bk == 0x7fffffff)
+                    for (int k = 0; k < nv && bk == 0x7fffffff; ++k)
+                        if (dist_at((Off)k * row + col) == T(INFINITY)) bk = k;
+            }
+
             // refinement from the closest recorded state, only where it can bring the wire within
             // its capture radius: from an interior state within the interior reach thin, from the
             // first or the last recorded state within a whole interval more than capth (the
@@ -898,6 +905,8 @@ __device__ __forceinline__ void group_wires_long(const F &f, const DcaArgs &a, c
                     nunc += 1 - conv;
                     d = residual<T>(tl, ii, D, lam, nin);
                 }
+            } else if (ALL && want) {
+                ((T *)a.dca_out)[(int64_t)(tl.w0 + ii) * S + s] = T(NAN);   // no state has a distance
             }
             if (used) acc.add_square(d);
         }

@@ -83,3 +83,34 @@ def test_sums_beside_a_track_that_is_not_finite(ctx, dtype, use_bounds, stride, 
     assert (np.abs(got["rss"][others] - ref["rss"]) <= rss_bound(e, lam, delta, dtype == torch.float32) + 1e-15).all()
     edge = (np.abs(e - lam) <= delta).sum(1)
     assert (np.abs(got["n_in"][others] - ref["n_in"]) <= edge).all() and (ref["n_in"] > 0).any()
+
+
+@pytest.mark.parametrize("dtype,far", [(torch.float32, 1e25), (torch.float64, 1e200)])
+@pytest.mark.parametrize("use_bounds", [False, True])
+@pytest.mark.parametrize("n_seeds,not_finite", [(1, None), (70, None), (70, 3), (70, 69)])
+def test_every_dca_of_a_track_without_distances(ctx, dtype, far, use_bounds, n_seeds, not_finite):
+    """A track whose squared distances overflow has its DCAs written when every DCA is wanted: infinite, as the
+    distance of its state is, and counted as not converged.  Where there is no distance at all they are NaN."""
+    ev = synth.multi_turn_event(1, counts=(4, 4, 4, 2))
+    spec = ev.partitions[0]
+    seeds = O.lattice(spec)[:n_seeds].copy()
+    seeds[0, :2] = far
+    if not_finite is not None:
+        seeds[not_finite, 3] = np.nan
+    bp = B.ScanParams(n_steps=ev.n_steps[0], stride=16, lam=1e-2)
+    field = B.DeviceField.from_synth(UNIFORM)
+    out = gpu_dca(ctx, field, bp, seeds, spec.charge, ev.wires, ev.hit_offsets, ev.drift, np.zeros(ev.n_hits, np.uint8),
+                  dtype, use_bounds=use_bounds)
+    assert out["n_unconv"] >= ev.n_wires and out["n_in"][0] == 0
+    dca = torch.full((ev.n_wires, n_seeds), -1.0, dtype=dtype, device="cuda")
+    again = torch.empty(n_seeds, dtype=dtype, device="cuda"), torch.empty(n_seeds, dtype=torch.int32, device="cuda")
+    B.comet_scan_dca(ctx, field, bp, out["pts"], out["nv"], out["charge"], out["w"], out["o"], out["d"], out["m"], *again,
+                     dca_out=dca, n_wires=ev.n_wires, bounds=out["bounds"])
+    dca = dca.double().cpu().numpy().T
+    assert np.array_equal(dca, out["dca"], equal_nan=True)
+    finite = np.arange(n_seeds) > 0
+    assert np.isposinf(dca[0]).all()
+    if not_finite is not None:
+        assert np.isnan(dca[not_finite]).all()
+        finite[not_finite] = False
+    assert (np.isfinite(dca[finite]) & (dca[finite] >= 0)).all()
