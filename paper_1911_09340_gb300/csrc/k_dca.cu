@@ -743,15 +743,17 @@ __device__ __forceinline__ void group_wires_long(const F &f, const DcaArgs &a, c
             // margin, the rounding of a distance.  A warp with a lane that does not meet this, or that is
             // not there after kSteps moves, scans the run.
             // The neighbours' distances are handed on where a scan of the run would have them, so both ways
-            // give the same bits.
+            // give the same bits.  A walk that leaves the run adds nothing: the run's closest state is then
+            // its boundary, farther than the state found, which is another run's to find or, in no run, is out
+            // of reach (and the boundary with it, unless it is the track's end: such a run is scanned).
             auto closest_in = [&](int ra, int rb, int kst) {
                 const int side = ALL ? 1 : 0;   // a scan of every state knows all neighbours
                 if constexpr (F::kAxial)
                     if (rb - ra >= kWalkMin<T>) {
-                        bool ok = true;
+                        bool ok = true, here = false;
                         T d0 = T(INFINITY), dm = T(INFINITY), dp = T(INFINITY);
                         int k = 0;
-                        if (want) {
+                        if (want && nv > ra) {
                             k = min(kst, nv - 1);
                             if (G1 > 1) {
                                 // the start is a segment's centre, several states from this lane's closest:
@@ -788,13 +790,14 @@ __device__ __forceinline__ void group_wires_long(const F &f, const DcaArgs &a, c
                                     dp = k < nv - 1 ? dist_at(o + row) : T(INFINITY);
                                 }
                             }
-                            const float far = dcv - a.h_rec_f * (float)(1 + max(0, max(k - min(ra, nv - 1), min(rb, nv - 1) - k)));
+                            const float far = dcv - a.h_rec_f * (float)(1 + max(k - ra, min(rb, nv - 1) - k));
                             const float hg = hg_k * dcv, f0 = (float)d0;
+                            here = k >= ra && k <= rb;
                             ok = !(dm <= d0 || dp < d0) && far > 0.f && f0 <= far * far &&
-                                 f0 * (a.margin_f * a.margin_f) <= hg * hg;
+                                 f0 * (a.margin_f * a.margin_f) <= hg * hg && (ALL || k >= ra || ra < nv - 1);
                         }
                         if (__all_sync(0xffffffffu, ok)) {
-                            if (want && (d0 < bd || (d0 == bd && k < bk))) {
+                            if (here && (d0 < bd || (d0 == bd && k < bk))) {
                                 bd = d0;
                                 bk = k;
                                 bdm = k > ra - side ? dm : T(INFINITY);

@@ -114,3 +114,35 @@ def test_every_dca_of_a_track_without_distances(ctx, dtype, far, use_bounds, n_s
         assert np.isnan(dca[not_finite]).all()
         finite[not_finite] = False
     assert (np.isfinite(dca[finite]) & (dca[finite] >= 0)).all()
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.float64])
+@pytest.mark.parametrize("stride,n_rec", [(1, 201), (1, 401), (2, 201)])
+def test_walk_into_another_run(ctx, dtype, stride, n_rec):
+    """Two bundles of nearly straight tracks cross at a wide angle beside a few wires.  The group's spheres
+    reach the wires before and after the crossing but not at it, so there are two runs of candidate
+    states, and each track's closest state lies in one of them: a search of the other run must not keep it
+    without its neighbours.  The sums are those of the scan of every state, bit for bit (each closest state
+    lies well inside its run)."""
+    rng = np.random.default_rng(n_rec)
+    h = 4e-3 / stride
+    S, ang = 32, np.deg2rad(65.0)
+    half = (n_rec - 1) * 4e-3 / 2
+    seeds = np.zeros((S, 6))
+    for s in range(S):
+        a = (ang if s % 2 else -ang) + (rng.normal() * 5e-4)
+        seeds[s] = [-half * np.cos(a), -half * np.sin(a), rng.normal() * 1e-3, 100 * np.cos(a), 100 * np.sin(a), 8.0]
+    hw = np.array([0.055, 0.058, 0.060, 0.062, 0.065])
+    wires = np.stack([np.zeros(5), -hw, np.zeros(5), np.zeros(5), np.zeros(5), np.ones(5)])
+    drift = hw * np.cos(ang)
+    bp = B.ScanParams(h=h, n_steps=(n_rec - 1) * stride, stride=stride, lam=4e-3, rmax=9.0, zmin=-9.0, zmax=9.0)
+    field = B.DeviceField.from_synth(synth.uniform_field(0.001))
+    run = lambda all_: gpu_dca(ctx, field, bp, seeds, -1, wires, np.arange(6), drift, np.zeros(5, np.uint8), dtype,
+                               want_dca=all_, use_bounds=not all_)
+    full, kept = run(True), run(False)
+    assert (full["n_in"] > 0).all()
+    for name in ("rss", "n_in"):
+        assert np.array_equal(full[name], kept[name])
+    with_spheres = gpu_dca(ctx, field, bp, seeds, -1, wires, np.arange(6), drift, np.zeros(5, np.uint8), dtype)
+    for name in ("dca", "rss", "n_in"):
+        assert np.array_equal(full[name], with_spheres[name])
