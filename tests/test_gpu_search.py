@@ -146,3 +146,29 @@ def test_walk_into_another_run(ctx, dtype, stride, n_rec):
     with_spheres = gpu_dca(ctx, field, bp, seeds, -1, wires, np.arange(6), drift, np.zeros(5, np.uint8), dtype)
     for name in ("dca", "rss", "n_in"):
         assert np.array_equal(full[name], with_spheres[name])
+
+
+@pytest.mark.parametrize("counts,stride", [((3, 5, 7, 9), 16), ((3, 5, 7, 9), 12), ((4, 4, 8, 3), 32)])
+def test_fp32_sums_over_tiles_of_wires(ctx, counts, stride):
+    """More wires than one tile holds, FP32 with one-state segments: each seed's counts are those of its wires
+    taken in three calls that fit one tile, and its RSS is their sum to the rounding of four FP32 results."""
+    ev = synth.multi_turn_event(1, counts=counts)
+    spec = ev.partitions[0]
+    wires, drift = [], []
+    for i in range(12):
+        other = synth.multi_turn_event(i, counts=counts)
+        wires.append(other.wires)
+        drift.append(other.drift[other.hit_offsets[:-1]])
+    wires, drift = np.concatenate(wires, 1)[:, :1100], np.concatenate(drift)[:1100]
+    assert wires.shape[1] == 1100
+    seeds = O.lattice(spec)
+    mask = (np.random.default_rng(2).random(1100) < 0.1).astype(np.uint8)
+    bp = B.ScanParams(n_steps=ev.n_steps[0], stride=stride, lam=1e-2, tol=1e-6)
+    field = B.DeviceField.from_synth(UNIFORM)
+    run = lambda a, b: gpu_dca(ctx, field, bp, seeds, spec.charge, wires[:, a:b], np.arange(b - a + 1), drift[a:b],
+                               mask[a:b], torch.float32, want_dca=False)
+    whole = run(0, 1100)
+    parts = [run(0, 500), run(500, 1000), run(1000, 1100)]
+    assert np.array_equal(whole["n_in"], sum(p["n_in"] for p in parts)) and (whole["n_in"] > 0).any()
+    assert whole["n_unconv"] == sum(p["n_unconv"] for p in parts)
+    assert np.allclose(whole["rss"], sum(p["rss"] for p in parts), rtol=4 * 2.0 ** -24, atol=0)
