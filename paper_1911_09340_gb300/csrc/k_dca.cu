@@ -58,8 +58,14 @@
 #ifndef COMET_DCA_MINB_FIELD
 #define COMET_DCA_MINB_FIELD 5
 #endif
-#ifndef COMET_DCA_U2
-#define COMET_DCA_U2 2
+// States per trip to memory of the long form's scan (11,475 seeds of an odd lattice x 275 states, FP32 axial:
+// 2 states 298 us, 4 206, 8 231; general uniform field, which has fewer registers free: 263, 4 237, 3 242,
+// but 2^14 seeds x 69 states, whose runs are short: 4 91, 3 89)
+#ifndef COMET_DCA_U
+#define COMET_DCA_U 4
+#endif
+#ifndef COMET_DCA_U_FIELD
+#define COMET_DCA_U_FIELD 3
 #endif
 // wires per chunk of the per-seed sums (the persistent kernel's finest work item)
 #ifndef COMET_DCA_CHUNK_W
@@ -643,7 +649,7 @@ __device__ __forceinline__ void group_wires_long(const F &f, const DcaArgs &a, c
     const int G0 = a.G0, G1 = a.G1;
     const int N1 = (G0 + G1 - 1) / G1;
     const Q4<T> *rec = tl.rec;
-    constexpr int kU = COMET_DCA_U2;
+    constexpr int kU = F::kAxial ? COMET_DCA_U : COMET_DCA_U_FIELD;
     const T kq2 = interior_margin<T, F>(f, a, gr);
     const uint32_t ends = end_segments<T>(a, gr, lane);
     // for the walk to the closest state (see below)
@@ -708,29 +714,56 @@ __device__ __forceinline__ void group_wires_long(const F &f, const DcaArgs &a, c
             auto dist_at = [&](Off o) {
                 return frame_dist2<T>(val(0, o), val(1, o), val(2, o), r0.x, r0.y, r0.z, r0.w, r1.x, r1.y, r1.z, r1.w);
             };
-            // every state of [k0, k1) of this lane's seed, kU at a time (span is warp-uniform); ranges come in
-            // ascending order, so an equal distance never replaces the one found
+            // every state of [k0, k1) of this lane's seed (span is warp-uniform); ranges come in ascending
+            // order, so an equal distance never replaces the one found
             auto scan = [&](int k0, int k1, int span) {
-                Off o = (Off)k0 * row + col;
                 T dprev = T(INFINITY);
                 bool last = false;   // the previous state is the closest so far
-                k1 = want ? k1 : 0;
-                for (int t0 = 0; t0 < span; t0 += kU, o += kU * row) {
-                    T d[kU];
-#pragma unroll
-                    for (int u = 0; u < kU; ++u) d[u] = k0 + t0 + u < k1 ? dist_at(o + u * row) : T(INFINITY);
-#pragma unroll
-                    for (int u = 0; u < kU; ++u) {
-                        const bool now = nearer<T>(d[u], bd);
-                        bdp = now ? T(INFINITY) : (last ? d[u] : bdp);
-                        if (now) {
-                            bdm = dprev;
-                            bd = d[u];
-                            bk = k0 + t0 + u;
-                        }
-                        dprev = d[u];
-                        last = now;
+                auto look = [&](int k, T d) {
+                    const bool now = nearer<T>(d, bd);
+                    bdp = now ? T(INFINITY) : (last ? d : bdp);
+                    if (now) {
+                        bdm = dprev;
+                        bd = d;
+                        bk = k;
                     }
+                    dprev = d;
+                    last = now;
+                };
+                k1 = want ? k1 : 0;
+                int k = k0;
+                Off o = (Off)k0 * row + col;
+                // kU at a time without a condition between their loads, so that they wait for memory once
+                // (past the lane's last state it is loaded again)
+                for (; span > 2; span -= kU, k += kU, o += kU * row) {
+                    const int left = k1 - k;
+                    T d[kU];
+                    if (left > 0) {
+                        T x[kU][3];
+                        Off ou = o;
+#pragma unroll
+                        for (int u = 0; u < kU; ++u) {
+#pragma unroll
+                            for (int c = 0; c < 3; ++c) x[u][c] = val(c, ou);
+                            if (u + 1 < left) ou += row;
+                        }
+#pragma unroll
+                        for (int u = 0; u < kU; ++u)
+                            d[u] = u < left ? frame_dist2<T>(x[u][0], x[u][1], x[u][2], r0.x, r0.y, r0.z, r0.w, r1.x, r1.y, r1.z, r1.w)
+                                            : T(INFINITY);
+                    } else {
+#pragma unroll
+                        for (int u = 0; u < kU; ++u) d[u] = T(INFINITY);
+                    }
+#pragma unroll
+                    for (int u = 0; u < kU; ++u) look(k + u, d[u]);
+                }
+                for (; span > 0; span -= 2, k += 2, o += 2 * row) {
+                    T d[2];
+#pragma unroll
+                    for (int u = 0; u < 2; ++u) d[u] = k + u < k1 ? dist_at(o + u * row) : T(INFINITY);
+#pragma unroll
+                    for (int u = 0; u < 2; ++u) look(k + u, d[u]);
                 }
             };
             // The closest state of a run [ra, rb] of candidate states.  Axial field: down the valley from a
