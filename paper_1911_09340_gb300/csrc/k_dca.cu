@@ -1155,6 +1155,18 @@ __host__ __device__ inline PLayout p_layout(int W, int es, int nsph)
 
 constexpr int kPersistMaxW = 1024;
 
+// Every DCA wanted: a group whose tracks all have fewer states than this is scanned without spheres, whose table
+// is not even loaded.  All tracks out of the region at once (with spheres, without): 2^14 seeds recorded for up
+// to 2,192 states 126 and 76 us, for 137 73 and 62, 59,535 seeds 194 and 182; with 3 to 22 states 2^14 seeds take
+// 92 us either way, above that the spheres are faster.
+constexpr int kFewForSpheres = 8;
+
+template <typename T, Search HOW>
+__device__ __forceinline__ bool use_spheres(const DcaArgs &a, const Group<T> &gr)
+{
+    return HOW != kAll || (a.bounds && gr.ehi + 1 >= kFewForSpheres);
+}
+
 // Resident CTAs per SM that the registers are allocated for.
 template <typename T, class F>
 constexpr int min_ctas(Search how)
@@ -1267,15 +1279,16 @@ __global__ void __launch_bounds__(kThreads, min_ctas<T, F>(HOW)) dca_persistent_
         const int64_t g = (int64_t)(it / (unsigned)nc);
         const int c = (int)(it % (unsigned)nc);
         const Group<T> gr = load_group<T>(a, g, lane);
+        const bool spheres = use_spheres<T, HOW>(a, gr);
         if (sph_smem) {
             build_spheres<T>(a, gr, lane, sph0, sph1, g);
-        } else if (L.nsph > 0) {
+        } else if (spheres) {
             // the usable part of this group's table from the recording kernel
             const float4 *src = (const float4 *)a.bounds + g * kBoundsPerGroup;
             for (int i = lane; i < L.nsph; i += 32) sph0[i] = __ldg(src + i);
             __syncwarp();
         }
-        const float4 *s0 = L.nsph > 0 ? sph0 : nullptr, *s1 = sph1;
+        const float4 *s0 = spheres ? sph0 : nullptr, *s1 = sph1;
         Acc<T> acc;
         int nin = 0;
         if (!split) {
@@ -1363,7 +1376,7 @@ __global__ void __launch_bounds__(kThreads, min_ctas<T, F>(HOW)) dca_tiled_kerne
     if (tid == 0) mbar_init(bar, 1);
     const int64_t g = (int64_t)blockIdx.x * kWarps + warp;
     const Group<T> gr = load_group<T>(a, g, lane);
-    const bool pruned = HOW != kAll || a.bounds;
+    const bool pruned = use_spheres<T, HOW>(a, gr);
     if (pruned) build_spheres<T>(a, gr, lane, sph0, sph1, g);
 
     const int W = a.W;

@@ -172,3 +172,23 @@ def test_fp32_sums_over_tiles_of_wires(ctx, counts, stride):
     assert np.array_equal(whole["n_in"], sum(p["n_in"] for p in parts)) and (whole["n_in"] > 0).any()
     assert whole["n_unconv"] == sum(p["n_unconv"] for p in parts)
     assert np.allclose(whole["rss"], sum(p["rss"] for p in parts), rtol=4 * 2.0 ** -24, atol=0)
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.float64])
+@pytest.mark.parametrize("above,stride,n_wires", [(-0.3, 16, 40), (1e-3, 16, 40), (2e-3, 16, 40), (1e-4, 1, 40), (1e-3, 16, 1030)])
+def test_every_dca_of_short_tracks(ctx, dtype, above, stride, n_wires):
+    """Tracks that leave the region after one to some tens of states: groups whose tracks all have a few states
+    are scanned, the others searched by their spheres, in either kernel, with the bits of the scan without spheres."""
+    ev = synth.multi_turn_event(1, counts=(7, 4, 8, 9))
+    spec = ev.partitions[0]
+    zmax = spec.centre[0] + above      # the fourth of the seven values of z0
+    seeds = O.lattice(spec)[576:1311]
+    wires = np.resize(np.arange(ev.n_wires), n_wires)
+    bp = B.ScanParams(n_steps=ev.n_steps[0], stride=stride, lam=1e-2, zmax=float(zmax))
+    drift = np.random.default_rng(1).uniform(0.0, 8e-3, n_wires)
+    full, kept = (gpu_dca(ctx, B.DeviceField.from_synth(UNIFORM), bp, seeds, spec.charge, ev.wires[:, wires],
+                          np.arange(n_wires + 1), drift, np.zeros(n_wires, np.uint8), dtype, use_bounds=b) for b in (False, True))
+    most = np.array([max(full["nv"].cpu().numpy()[i:i + 32]) for i in range(0, len(seeds), 32)])
+    assert (most < 8).any() and (above < 0 or ((most >= 8).any() and (most[most < 8] > 1).any()))
+    for name in ("dca", "rss", "n_in"):
+        assert np.array_equal(full[name], kept[name])
