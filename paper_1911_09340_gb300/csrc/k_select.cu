@@ -5,14 +5,13 @@
 // than the key chosen in round r-1".
 //
 // Pass 1: each block selects the k smallest keys of a contiguous chunk of the RSS array into the
-// scratch buffer.  Pass 2: one block selects among all blocks' candidates.  k = 1 is one block argmin
-// (per-thread minimum, warp-shuffle reduction, then a shared-memory reduction over the warps).  For
-// k > 1 every warp keeps the 64 smallest keys it has seen as a sorted list, two per lane: 64 keys at a
-// time are sorted by a bitonic network of shuffles and merged in, or skipped by one vote when none of
-// them precedes the list's k-th; the warps' lists are then merged pairwise through shared memory.  (k
-// rounds of a block argmin instead, each over the whole chunk and with three barriers, were bound by
-// the barriers' latency; both passes, k = 64: 2^14 FP32 seeds 206 -> 16 us, 2^18 FP32 478 -> 29 us, 2^18
-// FP64 2172 -> 48 us; k = 10 of 76,545 37 -> 18 us.)  Deterministic: no atomics, fixed networks.
+// scratch buffer.  Pass 2: one block selects among all blocks' candidates.  For the smallest k (select_how)
+// that is k rounds of a block argmin (per-thread minimum, warp-shuffle reduction, then a shared-memory
+// reduction over the warps), bound by the barriers' latency.  For larger k every warp keeps the 64 smallest
+// keys it has seen as a sorted list, two per lane: 64 keys at a time are sorted by a bitonic network of
+// shuffles and merged in, or skipped by one vote when none of them precedes the list's k-th; the warps'
+// lists are then merged pairwise through shared memory: 13 us for any k up to 64 and 59,535 FP32 seeds,
+// where 16 rounds take 52.  Deterministic: no atomics, fixed networks.
 #include <float.h>
 #include <stdint.h>
 
@@ -59,27 +58,37 @@ __device__ __forceinline__ Key<T> warp_min(Key<T> k)
     return k;
 }
 
-// Block argmin over the keys produced by get(j) for j in [0, n); thread 0 writes it.
-template <typename T, class Get>
-__device__ void block_min(int64_t n, Get get, T *out_v, int64_t *out_i)
+// k rounds of block argmin over the keys produced by get(j) for j in [0, n), each the smallest key after the
+// last round's (ONE: k = 1).  Thread 0 writes round r's key to out_v[r], out_i[r].
+template <typename T, bool ONE, class Get>
+__device__ void block_rounds(int64_t n, int k, Get get, T *out_v, int64_t *out_i)
 {
     __shared__ Key<T> red[kSelThreads / 32];
+    __shared__ Key<T> last;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    Key<T> best{T(0), kNone};
-    for (int64_t j = tid; j < n; j += kSelThreads) {
-        const Key<T> c = get(j);
-        if (key_less(c, best)) best = c;
-    }
-    best = warp_min(best);
-    if (lane == 0) red[wid] = best;
-    __syncthreads();
-    if (wid == 0) {
-        Key<T> b = lane < kSelThreads / 32 ? red[lane] : Key<T>{T(0), kNone};
-        b = warp_min(b);
-        if (lane == 0) {
-            *out_v = b.v;
-            *out_i = b.i;
+    for (int r = 0; r < (ONE ? 1 : k); ++r) {
+        [[maybe_unused]] Key<T> lk{T(0), -1};   // below every key
+        if constexpr (!ONE)
+            if (r > 0) lk = last;
+        Key<T> best{T(0), kNone};
+        for (int64_t j = tid; j < n; j += kSelThreads) {
+            const Key<T> c = get(j);
+            const bool later = ONE || lk.i < 0 || key_less(lk, c);
+            if (later && key_less(c, best)) best = c;
         }
+        best = warp_min(best);
+        if (lane == 0) red[wid] = best;
+        __syncthreads();
+        if (wid == 0) {
+            Key<T> b = lane < kSelThreads / 32 ? red[lane] : Key<T>{T(0), kNone};
+            b = warp_min(b);
+            if (lane == 0) {
+                out_v[r] = b.v;
+                out_i[r] = b.i;
+                if constexpr (!ONE) last = b;
+            }
+        }
+        if constexpr (!ONE) __syncthreads();
     }
 }
 
@@ -224,7 +233,23 @@ __device__ List64<typename SortKey<T>::type> block_smallest(int64_t n, int k, Va
     return best;
 }
 
+enum Select { kOne, kRounds, kLists };   // k = 1; a few rounds of block argmin; sorted lists
+
+constexpr int kMaxRounds = 3;
+constexpr int kSel2Threads = 1024;   // pass 2 over lists: one block, as many warps as it can have
+
+// Rounds are faster than the lists' sorting networks for the smallest k (rounds and lists, both passes,
+// 59,535 seeds: FP32 k = 2 8.2 and 13.1 us, 3 11.2 and 12.8, 4 13.8 and 12.0; FP64 k = 2 20.5 and 20.0,
+// but 256 seeds 11.0 and 12.7, 2^18 23.0 and 20.7).
 template <typename T>
+static Select select_how(int k, int n_blocks)
+{
+    if (k == 1) return kOne;
+    if (sizeof(T) == 4) return k <= kMaxRounds ? kRounds : kLists;
+    return k == 2 && n_blocks == 1 ? kRounds : kLists;
+}
+
+template <typename T, Select HOW>
 __global__ void __launch_bounds__(kSelThreads) select_pass1(const T *__restrict__ rss, int64_t S,
                                                             int k, T *pv, int64_t *pi)
 {
@@ -232,44 +257,43 @@ __global__ void __launch_bounds__(kSelThreads) select_pass1(const T *__restrict_
     const int64_t n = min((int64_t)kChunk, S - b0);
     pv += (int64_t)blockIdx.x * k;
     pi += (int64_t)blockIdx.x * k;
-    if (k == 1) {
-        block_min<T>(n, [&](int64_t j) { return Key<T>{rss[b0 + j], b0 + j}; }, pv, pi);
-        return;
-    }
-    const auto best = block_smallest<T, kSelThreads / 32>(n, k, [&](int64_t j) { return rss[b0 + j]; });
-    const int lane = threadIdx.x;
-    if (lane >= 32) return;
+    if constexpr (HOW != kLists) {
+        block_rounds<T, HOW == kOne>(n, k, [&](int64_t j) { return Key<T>{rss[b0 + j], b0 + j}; }, pv, pi);
+    } else {
+        const auto best = block_smallest<T, kSelThreads / 32>(n, k, [&](int64_t j) { return rss[b0 + j]; });
+        const int lane = threadIdx.x;
+        if (lane >= 32) return;
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        const int r = lane + 32 * h;
-        const uint32_t j = position(h ? best.b : best.a);
-        if (r < k) {
-            pv[r] = j < n ? rss[b0 + j] : T(0);
-            pi[r] = j < n ? b0 + j : kNone;
+        for (int h = 0; h < 2; ++h) {
+            const int r = lane + 32 * h;
+            const uint32_t j = position(h ? best.b : best.a);
+            if (r < k) {
+                pv[r] = j < n ? rss[b0 + j] : T(0);
+                pi[r] = j < n ? b0 + j : kNone;
+            }
         }
     }
 }
 
-constexpr int kSel2Threads = 1024;   // pass 2 with k > 1: one block, as many warps as it can have
-
-template <typename T, int NT>
-__global__ void __launch_bounds__(NT) select_pass2(const T *__restrict__ pv,
-                                                   const int64_t *__restrict__ pi, int64_t n, int k,
-                                                   int64_t *idx_out, T *rss_out)
+template <typename T, Select HOW>
+__global__ void __launch_bounds__(HOW == kLists ? kSel2Threads : kSelThreads)
+    select_pass2(const T *__restrict__ pv, const int64_t *__restrict__ pi, int64_t n, int k, int64_t *idx_out,
+                 T *rss_out)
 {
-    if constexpr (NT == kSelThreads) {
-        __shared__ T ov;
-        __shared__ int64_t oi;
-        block_min<T>(n, [&](int64_t j) { return Key<T>{pv[j], pi[j]}; }, &ov, &oi);
-        if (threadIdx.x == 0) {
-            *idx_out = oi;
-            if (rss_out) *rss_out = ov;
-        }
+    if constexpr (HOW != kLists) {
+        __shared__ T ov[kMaxRounds];
+        __shared__ int64_t oi[kMaxRounds];
+        block_rounds<T, HOW == kOne>(n, k, [&](int64_t j) { return Key<T>{pv[j], pi[j]}; }, ov, oi);
+        if (threadIdx.x == 0)   // which wrote them
+            for (int r = 0; r < (HOW == kOne ? 1 : k); ++r) {
+                idx_out[r] = oi[r];
+                if (rss_out) rss_out[r] = ov[r];
+            }
     } else {
         // places that pass 1 left empty (the last chunk shorter than k) stand after every candidate and
         // are never among the k <= S smallest; as NaN they sort after every number, and after every
         // NaN by their position
-        const auto best = block_smallest<T, NT / 32>(n, k, [&](int64_t j) {
+        const auto best = block_smallest<T, kSel2Threads / 32>(n, k, [&](int64_t j) {
             return pi[j] == kNone ? (T)NAN : pv[j];
         });
         const int lane = threadIdx.x;
@@ -300,7 +324,7 @@ __global__ void __launch_bounds__(kSelThreads) select_pass1_batch(BatchLaunch L)
     const T *__restrict__ rss = (const T *)a.rss;
     const int64_t b0 = lb * kChunk;
     const int64_t n = min((int64_t)kChunk, a.S - b0);
-    block_min<T>(n, [&](int64_t j) { return Key<T>{rss[b0 + j], b0 + j}; }, pv + lb, pi + lb);
+    block_rounds<T, true>(n, 1, [&](int64_t j) { return Key<T>{rss[b0 + j], b0 + j}; }, pv + lb, pi + lb);
 }
 
 template <typename T>
@@ -313,7 +337,7 @@ __global__ void __launch_bounds__(kSelThreads) select_pass2_batch(BatchLaunch L)
     const T *pv = (const T *)(pi + a.n_blocks);
     __shared__ T ov;
     __shared__ int64_t oi;
-    block_min<T>(a.n_blocks, [&](int64_t j) { return Key<T>{pv[j], pi[j]}; }, &ov, &oi);
+    block_rounds<T, true>(a.n_blocks, 1, [&](int64_t j) { return Key<T>{pv[j], pi[j]}; }, &ov, &oi);
     if (threadIdx.x == 0) {
         *a.idx_out = oi;
         if (a.rss_out) *(T *)a.rss_out = ov;
@@ -345,18 +369,25 @@ size_t select_scratch_bytes(comet_dtype dt, int64_t S, int k, int *n_blocks)
     return (size_t)nb * k * (es + sizeof(int64_t)) + 64;
 }
 
-template <typename T>
-static void sel_launch(const SelArgs &a, cudaStream_t st)
+template <typename T, Select HOW>
+static void sel_launch_how(const SelArgs &a, cudaStream_t st)
 {
     const int nb = a.n_blocks;
     int64_t *pi = (int64_t *)a.scratch;
     T *pv = (T *)(pi + (int64_t)nb * a.k);
-    select_pass1<T><<<nb, kSelThreads, 0, st>>>((const T *)a.rss, a.S, a.k, pv, pi);
-    const int64_t n = (int64_t)nb * a.k;
-    if (a.k == 1)
-        select_pass2<T, kSelThreads><<<1, kSelThreads, 0, st>>>(pv, pi, n, 1, a.idx_out, (T *)a.rss_out);
-    else
-        select_pass2<T, kSel2Threads><<<1, kSel2Threads, 0, st>>>(pv, pi, n, a.k, a.idx_out, (T *)a.rss_out);
+    select_pass1<T, HOW><<<nb, kSelThreads, 0, st>>>((const T *)a.rss, a.S, a.k, pv, pi);
+    select_pass2<T, HOW><<<1, HOW == kLists ? kSel2Threads : kSelThreads, 0, st>>>(pv, pi, (int64_t)nb * a.k, a.k,
+                                                                                  a.idx_out, (T *)a.rss_out);
+}
+
+template <typename T>
+static void sel_launch(const SelArgs &a, cudaStream_t st)
+{
+    switch (select_how<T>(a.k, a.n_blocks)) {
+    case kOne: sel_launch_how<T, kOne>(a, st); break;
+    case kRounds: sel_launch_how<T, kRounds>(a, st); break;
+    default: sel_launch_how<T, kLists>(a, st); break;
+    }
 }
 
 // Scratch of comet_scan_select_noalloc: one file-scope device array per device that loads the
@@ -388,7 +419,7 @@ cudaError_t static_select_scratch(void **ptr)
 cudaError_t kernel_binary_version(int *version)
 {
     cudaFuncAttributes fa;
-    const cudaError_t e = cudaFuncGetAttributes(&fa, select_pass1<float>);
+    const cudaError_t e = cudaFuncGetAttributes(&fa, select_pass1<float, kOne>);
     if (e == cudaSuccess) *version = fa.binaryVersion;
     return e;
 }

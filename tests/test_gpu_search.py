@@ -192,3 +192,26 @@ def test_every_dca_of_short_tracks(ctx, dtype, above, stride, n_wires):
     assert (most < 8).any() and (above < 0 or ((most >= 8).any() and (most[most < 8] > 1).any()))
     for name in ("dca", "rss", "n_in"):
         assert np.array_equal(full[name], kept[name])
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.float64])
+@pytest.mark.parametrize("S", [4, 5, 2047, 2048, 2049, 3 * 2048 + 2])
+@pytest.mark.parametrize("k", [1, 2, 3, 4])
+def test_top_k_by_rounds_or_lists(ctx, dtype, S, k):
+    """The smallest k by rounds of an argmin, larger ones by lists, against the oracle's order: one chunk, a last
+    chunk shorter than k, signed zeros (equal, so by index), infinities and NaN, ascending and descending input."""
+    rng = np.random.default_rng(S + k)
+    special = rng.choice(np.array([0.0, -0.0, np.inf, -np.inf, np.nan, 1.5, -2.0]), size=S)
+    few = np.full(S, np.nan)
+    few[rng.integers(S, size=2)] = 7.0
+    for v in (special, few, np.full(S, np.inf), np.arange(S, 0, -1.0), np.arange(S) * 1.0):
+        v = v.astype(np.float32 if dtype == torch.float32 else np.float64)
+        idx = torch.full((k,), -7, dtype=torch.int64, device="cuda")
+        val = torch.zeros(k, dtype=dtype, device="cuda")
+        B.comet_scan_select(ctx, torch.as_tensor(v, device="cuda"), k, idx, val)
+        order = np.lexsort((np.arange(S), np.where(np.isnan(v), 0.0, v), np.isnan(v)))[:k]
+        assert np.array_equal(idx.cpu().numpy(), order)
+        assert np.array_equal(val.cpu().numpy(), v[order], equal_nan=True)
+        only = torch.full((k,), -7, dtype=torch.int64, device="cuda")
+        B.comet_scan_select(ctx, torch.as_tensor(v, device="cuda"), k, only, None)
+        assert torch.equal(only, idx)
