@@ -297,7 +297,8 @@ __device__ __forceinline__ void advance_interval(const F &f, const PropArgs &a, 
 // stores), 2^14 x 2229 386 -> 160 us, 256 x 70 25 -> 15 us; FP64 2^15 x 139 427 -> 359 us.
 template <typename T, class F, int STRIDE, typename Off>
 __device__ __forceinline__ void record_inside(const F &f, const PropArgs &a, const AxialStep<T> &ks, T y[6],
-                                              bool valid, int64_t s, int lane, float4 *tab, T R0, T R1)
+                                              bool valid, int64_t s, int lane, float4 *tab, T R0, T R1,
+                                              bool together)
 {
     const int n_rec = a.n_rec, G0 = a.G0, G1 = a.G1;
     const int64_t plane = (int64_t)n_rec * a.S;
@@ -325,6 +326,13 @@ __device__ __forceinline__ void record_inside(const F &f, const PropArgs &a, con
     store();
     int r = 0;
     if (!tab) {
+        if (together) {
+            for (r = 1; r < n_rec; ++r) {
+                __syncthreads();
+                next();
+            }
+            return;
+        }
 #pragma unroll 4
         for (r = 1; r < n_rec; ++r) next();
         return;
@@ -469,12 +477,17 @@ __global__ void __launch_bounds__(128) propagate_kernel(F f, PropArgs a, BatchLa
         const AxialStep<float> kf{(float)ks.am1, (float)ks.b, (float)ks.c, (float)ks.d, (float)ks.dz};
         const bool in = stays_inside((float)y[0], (float)y[1], (float)y[2], (float)y[3], (float)y[4], kf, n_rec,
                                      a.lim_f[0], a.lim_f[1], a.lim_f[2], 4e-9f);
+        // Neighbouring warps share 32-byte sectors where a row is no multiple of 32 seeds.  Without spheres
+        // to form, the warps of a block drift apart and those sectors are written in halves; held side by
+        // side by a barrier per state (the block is all inside, so every warp takes this loop): 59,535 FP32
+        // seeds x 275 states 129 -> 98 us, 76,545 x 138 77 -> 56 us.  Whole lines gain nothing.
+        const bool together = !wb && (S & 31) != 0 && blockDim.x > 32 && __syncthreads_and(in);
         if (__all_sync(0xffffffffu, in)) {
             if (valid) a.n_valid[s] = n_rec;
             if (plane * (int64_t)sizeof(T) < ((int64_t)1 << 32))
-                record_inside<T, F, STRIDE, uint32_t>(f, a, ks, y, valid, s, lane, tab, R0, R1);
+                record_inside<T, F, STRIDE, uint32_t>(f, a, ks, y, valid, s, lane, tab, R0, R1, together);
             else
-                record_inside<T, F, STRIDE, size_t>(f, a, ks, y, valid, s, lane, tab, R0, R1);
+                record_inside<T, F, STRIDE, size_t>(f, a, ks, y, valid, s, lane, tab, R0, R1, together);
             return;
         }
     }

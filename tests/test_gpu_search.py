@@ -8,7 +8,7 @@ import oracle as O
 from paper_1911_09340_gb300 import binding as B
 from paper_1911_09340_gb300 import scan, synth
 
-from gpu_util import FP32_DCA_TOL, gpu_dca, per_wire_residual, rss_bound, seen
+from gpu_util import FP32_DCA_TOL, gpu_dca, gpu_propagate, per_wire_residual, rss_bound, seen
 
 pytestmark = pytest.mark.gpu
 UNIFORM = synth.uniform_field(1.0)
@@ -215,3 +215,28 @@ def test_top_k_by_rounds_or_lists(ctx, dtype, S, k):
         only = torch.full((k,), -7, dtype=torch.int64, device="cuda")
         B.comet_scan_select(ctx, torch.as_tensor(v, device="cuda"), k, only, None)
         assert torch.equal(only, idx)
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.float64])
+@pytest.mark.parametrize("n_seeds,stride,leaving", [(20001, 64, 0), (20001, 64, 3), (20031, 200, 1), (20000, 64, 0), (19999, 5000, 0)])
+def test_recording_side_by_side_equals_the_one_with_spheres(ctx, dtype, n_seeds, stride, leaving):
+    """Without spheres the warps of a block record side by side when the number of seeds is no multiple of 32: the
+    states and counts of the recording with spheres, in full blocks, in the last one (which has fewer warps), in
+    blocks with a track that leaves the region, and with a single recorded state."""
+    ev = synth.multi_turn_event(1, counts=(4, 4, 8, 4))
+    spec = ev.partitions[0]
+    seeds = np.resize(O.lattice(spec), (n_seeds, 6))
+    for s in np.linspace(40, n_seeds - 1, leaving).astype(int):
+        seeds[s, 3:] = [5.0, 0.0, 100.0]
+    bp = B.ScanParams(n_steps=ev.n_steps[0], stride=stride, zmin=-0.8, zmax=0.8)
+    field = B.DeviceField.from_synth(UNIFORM)
+    ctx.set_record_blocks(0)
+    try:
+        bounds = torch.empty(B.bounds_shape(n_seeds), dtype=torch.float32, device="cuda")
+        with_spheres = gpu_propagate(ctx, field, bp, seeds, spec.charge, dtype, bounds=bounds)
+        alone = gpu_propagate(ctx, field, bp, seeds, spec.charge, dtype)
+    finally:
+        ctx.set_record_blocks(1)
+    assert torch.equal(alone[3], with_spheres[3])
+    assert int((alone[3] < bp.n_rec).sum()) == (leaving if bp.n_rec > 1 else 0)
+    assert torch.equal(torch.nan_to_num(alone[2], nan=-1e3), torch.nan_to_num(with_spheres[2], nan=-1e3))
