@@ -240,3 +240,25 @@ def test_recording_side_by_side_equals_the_one_with_spheres(ctx, dtype, n_seeds,
     assert torch.equal(alone[3], with_spheres[3])
     assert int((alone[3] < bp.n_rec).sum()) == (leaving if bp.n_rec > 1 else 0)
     assert torch.equal(torch.nan_to_num(alone[2], nan=-1e3), torch.nan_to_num(with_spheres[2], nan=-1e3))
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.float64])
+@pytest.mark.parametrize("n_seeds,stride", [(1, 1), (33, 16), (70, 7), (5000, 32), (20001, 64)])
+def test_recording_in_a_uniform_field_of_any_direction(ctx, dtype, n_seeds, stride):
+    """Recorded without spheres (few seeds: a loop of its own) and with them: the same counts, and states that
+    agree to two ulp of the largest coordinate and momentum, also for tracks that leave the region."""
+    ev = synth.multi_turn_event(1, counts=(4, 4, 8, 4))
+    spec = ev.partitions[0]
+    seeds = np.resize(O.lattice(spec), (n_seeds, 6))
+    bp = B.ScanParams(n_steps=1600, stride=stride, zmin=-0.8, zmax=0.1, rmax=0.65)
+    field = B.DeviceField(0, b=(0.05, -0.1, 1.0))
+    bounds = torch.empty(B.bounds_shape(n_seeds), dtype=torch.float32, device="cuda")
+    a = gpu_propagate(ctx, field, bp, seeds, spec.charge, dtype, bounds=bounds)
+    b = gpu_propagate(ctx, field, bp, seeds, spec.charge, dtype)
+    assert torch.equal(a[3], b[3])
+    if n_seeds > 32:
+        assert int(a[3].min()) < bp.n_rec and int(a[3].max()) > 1
+    assert torch.equal(torch.isnan(a[2]), torch.isnan(b[2]))
+    diff = torch.nan_to_num(a[2] - b[2]).abs().amax((1, 2))
+    eps = torch.finfo(dtype).eps
+    assert float(diff[:3].max()) <= 2 * eps and float(diff[3:].max()) <= 2 * 128 * eps
