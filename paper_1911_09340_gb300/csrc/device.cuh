@@ -94,7 +94,7 @@ struct FieldTable {
     {
         constexpr float kOne = 12582912.f;
         const float r = __fadd_rd(g, kOne);
-        i = __float_as_int(r) - 0x4b400000;
+        i = (int)(__float_as_uint(r) - 0x4b400000u);   // (no overflow far outside, where it is not used)
         fi = __fsub_rn(r, kOne);
         t = __fsub_rn(g, (float)fi);
         return (unsigned)i < (unsigned)m;

@@ -262,3 +262,29 @@ def test_recording_in_a_uniform_field_of_any_direction(ctx, dtype, n_seeds, stri
     diff = torch.nan_to_num(a[2] - b[2]).abs().amax((1, 2))
     eps = torch.finfo(dtype).eps
     assert float(diff[:3].max()) <= 2 * eps and float(diff[3:].max()) <= 2 * 128 * eps
+
+
+@pytest.mark.parametrize("interleaved", [False, True])
+def test_fp32_cells_of_many_seeds(ctx, interleaved):
+    """More than two warps per scheduler take their cells by another lookup than a few seeds: the same track
+    points to 1 um of FP64, for tracks that leave the grid, enter it and run along its edge."""
+    half, n = 0.25, 11
+    g = np.linspace(-half, half, n)
+    z, y, x = np.meshgrid(g, g, g, indexing="ij")
+    table = np.stack([0.03 * z + 0.02 * y, 0.05 * x * z, 1.0 + 0.1 * x - 0.05 * y * z]).astype(np.float32)
+    field = B.DeviceField(1, table=table, origin=(-half,) * 3, spacing=2 * half / (n - 1), interleaved=interleaved)
+    start = [(0.0, 0.0, 0.0), (half, 0.0, 0.0), (-half, half, -half), (0.0, -half, half), (half + 0.01, 0.02, 0.0),
+             (g[n // 2], g[0], g[n // 2]), (-0.05, 0.04, -half - 0.02), (-3e6, 2e6, 3e6)]
+    few = np.array([[*p, 90.0 * np.cos(a), 90.0 * np.sin(a), 20.0] for p in start for a in (0.0, 1.3, 2.9, 4.4, 5.6)])
+    few = few.astype(np.float32).astype(np.float64)
+    bp = B.ScanParams(n_steps=400, stride=8, zmin=-9e9, zmax=9e9, rmax=9e9)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    many = np.resize(few, (256 * sms + 64, 6))
+    _, _, p32, n32 = gpu_propagate(ctx, field, bp, many, -1, torch.float32)
+    _, _, p64, n64 = gpu_propagate(ctx, field, bp, few, -1, torch.float64)
+    m = len(few)
+    assert torch.equal(n32[:m], n64) and torch.equal(n32[m:2 * m], n64)
+    near = torch.as_tensor(np.abs(few[:, 0]) < 1.0, device="cuda")
+    for c in (p32[:, :, :m], p32[:, :, m:2 * m]):
+        assert float((c[:3].double() - p64[:3])[:, :, near].abs().max()) < 1e-6
+        assert torch.equal(c[:3].isfinite(), p64[:3].isfinite())
