@@ -66,7 +66,8 @@ struct FieldUniform {
 };
 
 // Trilinear interpolation of a float32 table [3][nz][ny][nx]; coordinates clamped to the grid.
-template <typename T>
+// FAST: cells by cell_fast (float).
+template <typename T, bool FAST = false>
 struct FieldTable {
     static constexpr bool kAxial = false;
     const float *__restrict__ tab;
@@ -87,8 +88,9 @@ struct FieldTable {
 
     // The same for a float g inside a grid of m < 2^22 cells a side (false where it is not inside, or not
     // a number): the floor and its integer by adding 1.5 2^23, whose ulp is 1, rounded down, in place
-    // of the conversions (a quarter of the float rate here); no clamping is needed inside.  Recording in
-    // the tabulated field, 2^18 seeds x 2,204 steps: 7778 -> 7659 us (with the in-cell test as integers).
+    // of the conversions (a quarter of the float rate here); no clamping is needed inside.  It saves issue
+    // slots but its test lengthens the chain of one lookup: recording in the table x 69 states, conversions
+    // and this: 2^18 seeds 8154 and 8012 us, 2^16 2480 and 2402, 2^15 1530 and 1557, 2^14 1350 and 1417.
     // Not for single lookups (at): the DCA's refinement there went from 655 to 707 us, spilling.
     __device__ __forceinline__ static bool cell_fast(float g, int m, int &i, T &fi, T &t)
     {
@@ -157,7 +159,7 @@ struct FieldTable {
     {
         int ix, iy, iz;
         bool in = false;
-        if constexpr (sizeof(T) == 4) {
+        if constexpr (FAST) {
             const bool jx = cell_fast(gx, mx, ix, cc.fx, tx), jy = cell_fast(gy, my, iy, cc.fy, ty),
                        jz = cell_fast(gz, mz, iz, cc.fz, tz);
             in = jx && jy && jz;
@@ -255,10 +257,10 @@ struct FieldTable {
     }
 };
 
-template <typename T>
-inline FieldTable<T> make_table(const comet_field &f)
+template <typename T, bool FAST = false>
+inline FieldTable<T, FAST> make_table(const comet_field &f)
 {
-    return FieldTable<T>{(const float *)f.table, f.nx, f.ny, f.nz, (T)f.origin[0], (T)f.origin[1],
+    return FieldTable<T, FAST>{(const float *)f.table, f.nx, f.ny, f.nz, (T)f.origin[0], (T)f.origin[1],
                          (T)f.origin[2], (T)(1.0 / f.spacing), f.kind == 2 ? 1 : 0,
                          f.nx <= (1 << 22) ? f.nx - 1 : 0, f.ny <= (1 << 22) ? f.ny - 1 : 0,
                          f.nz <= (1 << 22) ? f.nz - 1 : 0};

@@ -782,8 +782,11 @@ static void prop_dispatch(const comet_field &f, const PropArgs &a, int stride, u
                                                stride, nb, L, st, nt);
         break;
     case FieldKind::Table:
-        prop_launch<T, FieldTable<T>, BATCH>(make_table<T>(f),
-                                             a, stride, nb, L, st, nt);
+        // FP32: cells by conversions up to two warps per scheduler, by cell_fast above (there)
+        if (sizeof(T) == 4 && (int64_t)nb * nt > (int64_t)device_sm_count() * 256)
+            prop_launch<T, FieldTable<T, sizeof(T) == 4>, BATCH>(make_table<T, sizeof(T) == 4>(f), a, stride, nb, L, st, nt);
+        else
+            prop_launch<T, FieldTable<T>, BATCH>(make_table<T>(f), a, stride, nb, L, st, nt);
         break;
     }
 }
