@@ -1767,6 +1767,8 @@ __global__ void __launch_bounds__(kThreads, COMET_DCA_BATCH_MINB) dca_batch_kern
             Acc<T> acc;
             int nin = 0;
             const int2 r = chunk_range(a.W, nc, k % nc);
+            // one form for every recording (an event's decides it, the launch is for all): runs of several states
+            // and FP64 are scanned where a launch of their own walks them, with the same bits
             group_wires<T, F, size_t, kShort>(f, a, gr, tl, s0, s0 + kN0Max, lane, acc, nin, nunc, r.x, r.y);
             ph[k * 32 + lane] = acc.hi;
             pl[k * 32 + lane] = acc.lo;

@@ -9,6 +9,7 @@ from paper_1911_09340_gb300 import binding as B
 from paper_1911_09340_gb300 import scan, synth
 
 from gpu_util import FP32_DCA_TOL, gpu_dca, gpu_propagate, per_wire_residual, rss_bound, seen
+from test_batch import _events, _reference
 
 pytestmark = pytest.mark.gpu
 UNIFORM = synth.uniform_field(1.0)
@@ -146,6 +147,101 @@ def test_walk_into_another_run(ctx, dtype, stride, n_rec):
     with_spheres = gpu_dca(ctx, field, bp, seeds, -1, wires, np.arange(6), drift, np.zeros(5, np.uint8), dtype)
     for name in ("dca", "rss", "n_in"):
         assert np.array_equal(full[name], with_spheres[name])
+
+
+@pytest.mark.parametrize("stride,cut", [(1, 40), (4, 40), (12, 33), (16, 64)])
+def test_byte_offsets_of_64_bits_equal_those_of_32(ctx, stride, cut):
+    """FP64 and every DCA wanted over a track array above 4 GiB (64-bit byte offsets) against its first seeds
+    alone (32-bit): the same states, sums and DCAs."""
+    ev = synth.multi_turn_event(1, counts=(16, 16, 32, 32))
+    spec = ev.partitions[0]
+    n_rec = ev.n_steps[0] // stride + 1
+    S = ((1 << 32) // (48 * n_rec) + 64) // 32 * 32
+    base = O.lattice(spec)
+    seeds = np.concatenate([base[:cut], np.resize(base[::97], (S - cut, 6))])
+    W = min(ev.n_wires, 12)
+    wires, offs = ev.wires[:, :W], ev.hit_offsets[: W + 1]
+    drift, mask = ev.drift[: offs[-1]], np.zeros(offs[-1], np.uint8)
+    bp = B.ScanParams(n_steps=ev.n_steps[0], stride=stride, lam=1e-2)
+    field = B.DeviceField.from_synth(UNIFORM)
+    ctx.set_record_blocks(0)
+    ctx.set_dca_chunk_wires(32)     # the sums' order depends on the number of seeds otherwise
+    try:
+        for want in (False, True):
+            big = gpu_dca(ctx, field, bp, seeds, spec.charge, wires, offs, drift, mask, torch.float64, want_dca=want)
+            n32 = cut // 32 * 32
+            small = gpu_dca(ctx, field, bp, seeds[:n32], spec.charge, wires, offs, drift, mask, torch.float64, want_dca=want)
+            assert 48 * n_rec * S >= 1 << 32
+            for name in ("rss", "n_in") + (("dca",) if want else ()):
+                assert np.array_equal(big[name][:n32], small[name])
+            assert torch.equal(big["pts"][:, :, :n32], small["pts"])
+            del big, small
+    finally:
+        ctx.set_record_blocks(1)
+        ctx.set_dca_chunk_wires(0)
+
+
+@pytest.mark.parametrize("dtype_name", ["float32", "float64"])
+@pytest.mark.parametrize("stride", [1, 4])
+def test_batch_of_long_recordings_equals_per_event_scan(ctx, dtype_name, stride):
+    """More than 192 recorded states (level-1 segments of several states): the batched launches scan the runs
+    of candidate states that the single-event launches walk, with the same bits."""
+    from paper_1911_09340_gb300 import batch
+    dtype = getattr(torch, dtype_name)
+    events = _events(5)
+    ctx.set_record_blocks(0)
+    try:
+        ref = _reference(ctx, events, dtype, stride)
+        bs = batch.BatchScanner(ctx, dtype, stride=stride, lam=1e-2, slots=3, max_seeds=4096, max_total_seeds=1 << 13,
+                                max_wires=512, max_hits=1024)
+        r = bs.run(events, collect=True)
+    finally:
+        ctx.set_record_blocks(1)
+    for rr, res in zip(ref, r["results"]):
+        for p, part in enumerate(rr):
+            assert res.best_idx[p] == part["idx"] and res.best_rss[p] == part["rss"]
+            assert np.array_equal(res.hit_class[p], part["hit_class"])
+
+
+@pytest.mark.parametrize("fault,step", [("k0", 3), ("k65", 3), ("k_above_S", 3), ("no_idx", 3), ("no_rss", 2), ("no_class", 4),
+                                        ("no_points", 1)])
+def test_partition_call_refuses_what_its_steps_refuse(ctx, fault, step):
+    """comet_scan_partition ends at the step that refuses its arguments, with that step's status; the results
+    of the later steps stay as they were, and the context serves the next call."""
+    ev = synth.multi_turn_event(1, counts=(2, 3, 2, 2))
+    spec = ev.partitions[0]
+    S = spec.n_seeds
+    bp = B.ScanParams(n_steps=ev.n_steps[0], stride=16, lam=1e-2)
+    dev = scan.DeviceEvent.from_event(ev)
+    field = B.DeviceField.from_synth(UNIFORM)
+
+    def call(k=2, **kw):
+        ws = scan.Workspace(S, bp.n_rec, ev.n_hits, k=64)
+        ws.idx.fill_(-7), ws.hit_class.fill_(9), ws.rss.fill_(-3.0)
+        a = dict(seeds=ws.seeds, charge=ws.charge, points=ws.points, n_valid=ws.n_valid, bounds=ws.bounds, wires=dev.wires,
+                 hit_offsets=dev.hit_offsets, drift=dev.drift, hit_mask=dev.mask, rss=ws.rss, n_in=ws.n_in, idx=ws.idx,
+                 best=ws.best, hit_class=ws.hit_class, n_wires=dev.W)
+        a.update(kw)
+        try:
+            B.comet_scan_partition(ctx, field, bp, spec, k, **a)
+            failed = False
+        except B.CometError as e:
+            failed = True
+            assert e.status == 1
+        torch.cuda.synchronize()
+        return failed, ws
+    kw = {"k0": dict(k=0), "k65": dict(k=65), "k_above_S": dict(k=S + 1), "no_idx": dict(idx=None), "no_rss": dict(rss=None),
+          "no_class": dict(hit_class=None),
+          "no_points": dict(points=None)}[fault]
+    failed, ws = call(**kw)
+    assert failed and bool((ws.hit_class == 9).all())
+    if step <= 3:
+        assert bool((ws.idx == -7).all())
+    if step <= 2:
+        assert bool((ws.rss == -3.0).all())
+    (ok_a, a), (ok_b, b) = call(), call()
+    assert not ok_a and not ok_b and torch.equal(a.idx, b.idx) and torch.equal(a.rss[:S], b.rss[:S])
+    assert a.idx[:2].tolist() == np.argsort(a.rss[:S].cpu().numpy(), kind="stable")[:2].tolist()
 
 
 @pytest.mark.parametrize("counts,stride", [((3, 5, 7, 9), 16), ((3, 5, 7, 9), 12), ((4, 4, 8, 3), 32)])
