@@ -60,7 +60,8 @@
 #endif
 // States per trip to memory of the long form's scan (11,475 seeds of an odd lattice x 275 states, FP32 axial:
 // 2 states 298 us, 4 206, 8 231; general uniform field, which has fewer registers free: 263, 4 237, 3 242,
-// but 2^14 seeds x 69 states, whose runs are short: 4 91, 3 89)
+// but 2^14 seeds x 69 states, whose runs are short: 4 91, 3 89).  FP64 waits for its pipe, not for memory: 2, or 4 when
+// every DCA is wanted (2^15 seeds x 137 states 2 1517, 4 1555; every DCA of 256 x 137 without spheres 457 and 403)
 #ifndef COMET_DCA_U
 #define COMET_DCA_U 4
 #endif
@@ -649,7 +650,7 @@ __device__ __forceinline__ void group_wires_long(const F &f, const DcaArgs &a, c
     const int G0 = a.G0, G1 = a.G1;
     const int N1 = (G0 + G1 - 1) / G1;
     const Q4<T> *rec = tl.rec;
-    constexpr int kU = F::kAxial ? COMET_DCA_U : COMET_DCA_U_FIELD;
+    constexpr int kU = sizeof(T) == 8 && !ALL ? 2 : F::kAxial ? COMET_DCA_U : COMET_DCA_U_FIELD;
     const T kq2 = interior_margin<T, F>(f, a, gr);
     const uint32_t ends = end_segments<T>(a, gr, lane);
     // for the walk to the closest state (see below)
