@@ -27,7 +27,8 @@
 // and the last recorded state the refinement reaches up to h_rec (not h_rec/2) from the nearest
 // recorded state, so segments that may hold a track end are tested, and an end state refined,
 // within capture radius + h_rec.  With dca_out (exact DCA for every wire) the spheres leave the segments
-// that may hold a lane's closest state; without a sphere table every state is then scanned.
+// that may hold a lane's closest state; without a sphere table, or where a group's tracks all have a few
+// states, every state is then scanned.
 //
 // RSS: each thread sums its wires' d_i^2 in ascending wire order within each wire chunk (FP32 as a
 // TwoSum pair, FP64 plainly), then the chunks' sums in chunk order.  Atomics only hand out work
@@ -49,7 +50,7 @@
 #define COMET_DCA_MINB_LONG 6
 #endif
 // FP64: bound by the FP64 pipe rather than by resident warps; fewer CTAs per SM buy registers (at
-// 72 the FP64 kernels spill ~300 B per thread; 4 CTAs 974 us, 3 CTAs 961 at 2^15 x 139 states)
+// 72 the FP64 kernels spill ~300 B per thread; 4 CTAs take 1% longer than 3 at 2^15 x 139 states)
 #ifndef COMET_DCA_MINB_F64
 #define COMET_DCA_MINB_F64 3
 #endif
@@ -453,8 +454,8 @@ __device__ __forceinline__ T residual(const Tile<T> &tl, int ii, T D, T lam, int
 
 // Shorter runs are scanned one state after the other with its momentum, longer ones two positions at a
 // time and the momentum of the closest state loaded at the end (group_wires_short).  Recordings of 32 mm
-// give runs of 1.5 states, of 16 mm up to 13 (an odd lattice's wide groups): 2^18 x 70 states 445 us
-// in pairs with momentum, 449 us so; 76,545 x 139 (odd lattice) 569 and 514 us, all one by one 675 us.
+// give runs of 1.5 states, where both ways cost the same; of 16 mm up to 13 in an odd lattice's wide
+// groups: 76,545 seeds x 139 states all one by one 675 us, in pairs with momentum 569, so 514.
 constexpr int kFewStates = 4;
 
 // Runs of more than this many states are walked, not scanned (group_wires_long): a walk looks at about
@@ -469,10 +470,9 @@ constexpr int kWalkMin = sizeof(T) == 4 ? 10 : 4;
 // positions only, runs of many states walked, and the search bounded by the spheres when every DCA
 // is wanted.  The short form is bound by instruction issue (72% of it used at 2^18 seeds), the refinement
 // taking about half; the long one by the latency of the walk's loads in FP32, by the FP64 pipe in FP64.
-// Before (one form, 64-bit addresses, momentum selected along) and now, FP32: 2^18 seeds x 70 states
-// 463 -> 425 us (449 before refine_dca's single exit), 76,545 x 139 592 -> 510, 2^14 x 2,229 560 -> 156, every
-// DCA of 2^14 x 70 373 -> 102; FP64: 4,096 x 2,229 808 -> 245, 2^15 x 139 1415 -> 963 (280 and 1210
-// before refine_dca's shorter iteration and the comparisons off the FP64 pipe).
+// One form for all, with 64-bit addresses and momenta, and these, FP32: 2^18 seeds x 70 states 463 and 425 us,
+// 76,545 x 139 592 and 510, 2^14 x 2,229 560 and 156, every DCA of 2^14 x 70 373 and 98; FP64: 4,096 x 2,229
+// 808 and 245, 2^15 x 139 1415 and 970.
 // Off: the byte offset of a recorded value, 32 bits when the track array is small enough.
 template <typename T, class F, typename Off>
 __device__ __forceinline__ void group_wires_short(const F &f, const DcaArgs &a, const Group<T> &gr,

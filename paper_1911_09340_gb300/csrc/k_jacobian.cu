@@ -8,17 +8,16 @@
 // derivatives in one variable, |p|: the path is carried as X and P, each with its derivative in ln(1/|p|)
 // (forward mode), and the chain rule in (z0, phi, pz, pT) is applied once, at its end.  This part's FP64
 // unit holds its scheduler for 64 cycles per warp instruction, whatever the active lanes, so the
-// kernel's time is its longest lane's count of FP64 instructions: carrying four derivatives through
-// every step and through the maps' powers took 225 us for 16 seeds x 100 wires.  A whole call, 16 seeds x
-// 134 wires x 138 states 438 -> 95 us, 64 x 134 x 2229 584 -> 232 us, 1000 x 134 x 138 1856 -> 663 us.
+// kernel's time is its longest lane's count of FP64 instructions.  A whole call with four derivatives
+// carried through every step and through the maps' powers, and so: 16 seeds x 134 wires x 138 states
+// 438 and 95 us, 64 x 134 x 2229 584 and 232, 1000 x 134 x 138 1856 and 663.
 //
 // The DCA of a wire is the distance at the point of closest approach (PCA) found as in the scan: the
 // closest recorded state (searched in FP32, settled in FP64 among its neighbours), then the local
 // virtual-plane Newton refinement of Algorithm 2, each refinement step being one RK4 step of the
-// axial map.  At the PCA the distance
-// is stationary along the track, so dD/dtheta = nhat . dx/dtheta at the fixed arc length of the PCA
-// (envelope theorem): the refinement steps enter the product of maps with their lengths held fixed.
-// nhat is the unit vector from the wire to the PCA.
+// axial map.  At the PCA the distance is stationary along the track, so dD/dtheta = nhat . dx/dtheta at
+// the fixed arc length of the PCA (envelope theorem): the refinement steps enter the product of maps with
+// their lengths held fixed.  nhat is the unit vector from the wire to the PCA.
 //
 // Smoothed residual (Eq. 1 with a differentiable cap): e = min_j |D - r_j| over the wire's unmasked
 // hits, w = sigmoid((lambda - e) / tau), term = w e^2 + (1 - w) lambda^2.  Gauss-Newton treats w as

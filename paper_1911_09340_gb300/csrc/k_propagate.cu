@@ -92,9 +92,8 @@ __global__ void __launch_bounds__(256) lattice_kernel(LatArgs a, const __grid_co
 #pragma unroll
     for (int d = 1; d < 3; ++d) b[d] = a.counts[d] % 4 == 0 ? 4 : (a.counts[d] % 2 == 0 ? 2 : 1);
     b[3] = 1;
-    // The block's and the node's indices by divisions: by the powers of two b with shifts, of the block in
-    // 32 bits where it fits (nine divisions of
-    // 64 bits before: 2^18 seeds 7.6 -> 6.6 us, a batch's 34 lattices 414 -> 328).
+    // The block's and the node's indices: the divisions by b, powers of two, are shifts, those of the block's
+    // number are in 32 bits where it fits (with nine divisions of 64 bits 2^18 seeds took 7.6 us, so 6.6).
     const int sh[4] = {b[0] >> 1, b[1] >> 1, b[2] >> 1, 0};   // log2 of b
     const int vsh = sh[0] + sh[1] + sh[2];
     unsigned in = (unsigned)s & ((1u << vsh) - 1u);
@@ -292,9 +291,10 @@ __device__ __forceinline__ void advance_interval(const F &f, const PropArgs &a, 
 // (one addition per state then serves the six stores).  With one-state segments two states are recorded
 // before their two spheres are formed, so that the two chains of shuffles and reductions overlap (a
 // few seeds leave one warp per scheduler, which has nothing else to issue).  Bound by the stores at
-// 2^18 seeds and by the issue of one warp per scheduler at a few thousand.  FP32 with spheres, before
-// (the general loop of propagate_kernel) and after: 2^18 seeds x 70 states 101 -> 82 us (5.2 TB/s of
-// stores), 2^14 x 2229 386 -> 160 us, 256 x 70 25 -> 15 us; FP64 2^15 x 139 427 -> 359 us.
+// 2^18 seeds and by the issue of one warp per scheduler at a few thousand.  The general loop of
+// propagate_kernel and this, FP32 with spheres: 2^18 seeds x 70 states 101 and 82 us (5.2 TB/s of stores),
+// 2^14 x 2229 386 and 160, 256 x 70 25 and 15; FP64 2^15 x 139 427 and 248.
+// together: the block's warps take a state at a time side by side (see propagate_kernel).
 template <typename T, class F, int STRIDE, typename Off>
 __device__ __forceinline__ void record_inside(const F &f, const PropArgs &a, const AxialStep<T> &ks, T y[6],
                                               bool valid, int64_t s, int lane, float4 *tab, T R0, T R1,
@@ -417,7 +417,7 @@ template <typename T>
 constexpr bool is_uniform<FieldUniform<T>> = true;
 
 // BATCH: one launch for a batch of events; block b belongs to the event that batch_find gives.
-// Lanes past the last seed repeat it without storing: with idle lanes instead, the shuffles of every
+// Lanes past the last seed repeat it (in a uniform axial field without storing): with idle lanes instead, the shuffles of every
 // sphere found the last warp of a seed count that is no multiple of 32 diverged, and that one warp
 // made the launch 4 times as long (10,000 seeds x 140 states: 191 us against 46 us for 9,984).
 template <typename T, class F, int STRIDE, bool BATCH>

@@ -9,8 +9,8 @@
 // then walks them in order: lane j holds accepted reference j, so each candidate costs one lane-parallel
 // test and one vote.  The test is decided in float where the float difference clears the width by more
 // than its rounding, in double only otherwise (this part's double rate is 1/64 of its float rate).  One
-// warp doing everything in double, a candidate at a time: 64 candidates of the iterative scan's coarse
-// lattice 165 us, now 13; 1,000 spread ones 709 -> 89 us.  phi differences are taken modulo 2 pi.
+// warp doing everything in double, a candidate at a time, and this: 64 candidates of the iterative scan's
+// coarse lattice 165 and 13 us, 1,000 spread ones 709 and 89.  phi differences are taken modulo 2 pi.
 #include <math.h>
 
 #include "device.cuh"
