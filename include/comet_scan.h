@@ -184,8 +184,8 @@ comet_status comet_scan_lattice(comet_ctx *ctx, comet_dtype dtype, const comet_l
  *   bounds   optional out (NULL to skip), [ceil(S/32)][200][4] float32, 16-byte aligned: search
  *            bounds for comet_scan_dca with the same params -- for each group of 32 consecutive
  *            seeds, the bounding spheres (x, y, z, radius) of its track segments (8 super-segments,
- *            24 level-1 segments each; a negative radius marks a segment no seed has, an infinite one
- *            a segment of a group with a track that is not finite).  Writing them costs a few percent of this call and saves
+ *            24 level-1 segments each; a negative radius marks a segment no seed has, one that is not
+ *            a number a segment of a group with a track that is not finite).  Writing them costs a few percent of this call and saves
  *            comet_scan_dca from rebuilding them.
  * One thread extrapolates one seed with fixed-step RK4.  The FP32 path carries each state component
  * as an unevaluated float pair (a compensated sum), so that 6,500 steps stay within a few um of FP64;

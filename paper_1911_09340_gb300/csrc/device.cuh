@@ -313,8 +313,7 @@ __device__ __forceinline__ void axial_increment(const AxialStep<T> &k, const T y
 // z moves by dz per interval.  Tested in float whatever the working precision: the margins (0.1 mm,
 // per_state for each state's rounding and 2e-6 of the coordinates; |M|^k from |M|^2 - 1 plus its
 // rounding) are far above the float rounding here and the rounding of the recorded states.  A track near
-// the boundary, a straight one (M = 1), one that is not finite or one whose squared coordinates would
-// overflow a float (the margin grows with them) keeps the per-state test.
+// the boundary, a straight one (M = 1) or one that is not finite keeps the per-state test.
 __device__ __forceinline__ bool stays_inside(float x, float y, float z, float px, float py,
                                              const AxialStep<float> &k, int n_rec, float zmin, float zmax,
                                              float rmax2, float per_state)
@@ -331,7 +330,7 @@ __device__ __forceinline__ bool stays_inside(float x, float y, float z, float px
     float rout = sqrtf(cx * cx + cy * cy) + rr * (1.f + 1.1f * grow);
     const float margin = 1e-4f + per_state * n + 2e-6f * (rout + fabsf(z) + fabsf(z1));
     rout += margin;
-    return margin < 1e9f && rout * rout < rmax2 && fminf(z, z1) > zmin + margin && fmaxf(z, z1) < zmax - margin;
+    return rout * rout < rmax2 && fminf(z, z1) > zmin + margin && fmaxf(z, z1) < zmax - margin;
 }
 
 // The four stages of one classic RK4 step of length h from state y, the field from look(x, y, z,
@@ -734,19 +733,14 @@ __device__ __forceinline__ float4 spread_sphere(const WarpSpread<T> &w, T reach)
     return make_float4((float)(T(0.5) * w.sx), (float)(T(0.5) * w.sy), (float)(T(0.5) * w.sz), rad);
 }
 
-// The warp's bounding sphere of one segment; radius < 0 when no lane has the segment.  With a track in the
-// group that is not finite, or so far away that the distance tests in float would overflow, no sphere
-// bounds the segment: an infinite one about the origin, which excludes nothing.  (Tracks that provably
-// stay inside the region are finite and nearer than that, so record_inside forms its spheres without
-// this test: with it, recording 2^18 FP32 seeds x 69 states took 100 us instead of 95.)
+// The warp's bounding sphere of one segment; radius < 0 when no lane has the segment, not a number when a
+// track of the group is not finite (such a sphere excludes nothing: sphere_within).
 template <typename T>
 __device__ __forceinline__ float4 warp_sphere(bool has, T x, T y, T z, T reach)
 {
     const uint32_t hm = __ballot_sync(0xffffffffu, has);
     if (hm == 0u) return make_float4(0.f, 0.f, 0.f, -1.f);
-    const float4 sp = spread_sphere<T>(warp_spread<T>(has, __ffs(hm) - 1, 31 - __clz(hm), x, y, z), reach);
-    const bool bounded = fabsf(sp.x) + fabsf(sp.y) + fabsf(sp.z) + sp.w < 1e18f;
-    return bounded ? sp : make_float4(0.f, 0.f, 0.f, INFINITY);
+    return spread_sphere<T>(warp_spread<T>(has, __ffs(hm) - 1, 31 - __clz(hm), x, y, z), reach);
 }
 
 // ------------------------------------------------------------------------------------------------

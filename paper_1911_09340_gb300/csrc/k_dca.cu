@@ -313,12 +313,13 @@ __device__ __forceinline__ float sphere_margin(float av, float aw)
     return sizeof(T) == 4 ? 0.f : sph_margin_f32(av, aw);
 }
 
-// Whether the sphere reaches within lim of the wire; d2 = the squared distance of its centre.
+// Whether the sphere reaches within lim of the wire; d2 = the squared distance of its centre.  A comparison
+// that is not a number does not exclude: the spheres of a group with a track that is not finite hold it.
 __device__ __forceinline__ bool sphere_within(const float4 &sp, const float4 &v, const float4 &w, float lim, float &d2)
 {
     d2 = frame_dist2<float>(sp.x, sp.y, sp.z, v.x, v.y, v.z, v.w, w.x, w.y, w.z, w.w);
     const float l = lim + sp.w;
-    return sp.w >= 0.f && d2 <= l * l;
+    return !(sp.w < 0.f) && !(d2 > l * l);
 }
 
 // Capture radius and frame of wire i of a staged tile (one thread per wire), packed with its
