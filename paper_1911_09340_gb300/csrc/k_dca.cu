@@ -633,7 +633,7 @@ __device__ __forceinline__ void group_wires_short(const F &f, const DcaArgs &a, 
     }
 }
 
-template <typename T, class F, typename Off, bool ALL>
+template <typename T, class F, typename Off, bool ALL, bool WIDE>
 __device__ __forceinline__ void group_wires_long(const F &f, const DcaArgs &a, const Group<T> &gr,
                                             const Tile<T> &tl, const float4 *sph0,
                                             const float4 *sph1, int lane, Acc<T> &acc, int &nin,
@@ -737,7 +737,7 @@ __device__ __forceinline__ void group_wires_long(const F &f, const DcaArgs &a, c
                 Off o = (Off)k0 * row + col;
                 // kU at a time without a condition between their loads, so that they wait for memory once
                 // (past the lane's last state it is loaded again)
-                for (; span > 2; span -= kU, k += kU, o += kU * row) {
+                for (; WIDE && span > 2; span -= kU, k += kU, o += kU * row) {
                     const int left = k1 - k;
                     T d[kU];
                     if (left > 0) {
@@ -952,7 +952,7 @@ __device__ __forceinline__ void group_wires_long(const F &f, const DcaArgs &a, c
 }
 
 // How a launch searches for the closest states.
-enum Search { kShort, kLong, kAll };   // runs of a few states; runs of many; every DCA wanted
+enum Search { kShort, kFew, kLong, kAll };   // runs of a few states (two ways); runs of many; every DCA wanted
 
 template <typename T, class F, typename Off, Search HOW>
 __device__ __forceinline__ void group_wires(const F &f, const DcaArgs &a, const Group<T> &gr,
@@ -963,7 +963,7 @@ __device__ __forceinline__ void group_wires(const F &f, const DcaArgs &a, const 
     if constexpr (HOW == kShort)
         group_wires_short<T, F, Off>(f, a, gr, tl, sph0, sph1, lane, acc, nin, nunc, wb, we);
     else
-        group_wires_long<T, F, Off, HOW == kAll>(f, a, gr, tl, sph0, sph1, lane, acc, nin, nunc, wb, we);
+        group_wires_long<T, F, Off, HOW == kAll, HOW != kFew>(f, a, gr, tl, sph0, sph1, lane, acc, nin, nunc, wb, we);
 }
 
 // Wire chunk c of n over W wires: [c * wc, min((c + 1) * wc, W)), wc = ceil(W / n).
@@ -1539,15 +1539,24 @@ static cudaError_t dca_launch_how(const F &fld, const DcaArgs &a, cudaStream_t s
                : dca_launch_off<T, F, size_t, HOW>(fld, a, st);
 }
 
+template <class F>
+constexpr bool is_general = false;
+template <typename T>
+constexpr bool is_general<FieldUniform<T>> = true;
+
 // FP32 in an axial field takes the short form (group_wires_short) when a level-1 segment is one state:
 // runs are then a few states long.  In the tiled kernel too (long and short form): 2^16 seeds x 69 states x
 // 1,100 wires 605 and 574 us, 11,475 seeds of an odd lattice x 138 states x 1,100 wires 3,043 and 2,097 us.
+// In a general uniform field it takes the long form without the wide scan then (with and without, 2^14 seeds x 69
+// states 88 and 82 us, 2^18 804 and 718; a table's refinement takes so long that it makes no difference).
 template <typename T, class F>
 static cudaError_t dca_launch(const F &fld, const DcaArgs &a, cudaStream_t st)
 {
     if (a.exact_all) return dca_launch_how<T, F, kAll>(fld, a, st);
     if constexpr (sizeof(T) == 4 && F::kAxial)
         if (a.G1 == 1) return dca_launch_how<T, F, kShort>(fld, a, st);
+    if constexpr (sizeof(T) == 4 && is_general<F>)
+        if (a.G1 == 1) return dca_launch_how<T, F, kFew>(fld, a, st);
     return dca_launch_how<T, F, kLong>(fld, a, st);
 }
 
