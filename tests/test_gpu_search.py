@@ -384,3 +384,22 @@ def test_fp32_cells_of_many_seeds(ctx, interleaved):
     for c in (p32[:, :, :m], p32[:, :, m:2 * m]):
         assert float((c[:3].double() - p64[:3])[:, :, near].abs().max()) < 1e-6
         assert torch.equal(c[:3].isfinite(), p64[:3].isfinite())
+
+
+@pytest.mark.parametrize("use_bounds", [False, True])
+@pytest.mark.parametrize("counts,stride", [((4, 4, 4, 2), 16), ((3, 5, 3, 7), 16), ((3, 5, 3, 7), 8), ((1, 1, 1, 1), 32)])
+def test_fp32_sums_in_a_uniform_field_of_any_direction(ctx, use_bounds, counts, stride):
+    """Segments of one state (short and long runs) and of several against the oracle, within the DCA bars' bound."""
+    ev = synth.multi_turn_event(1, counts=counts)
+    spec = ev.partitions[0]
+    f32 = torch.float32
+    seeds, wires, drift, lam = seen(O.lattice(spec), f32), seen(ev.wires, f32), seen(ev.drift, f32), 1e-2
+    mask = np.zeros(ev.n_hits, np.uint8)
+    b = tuple(seen((0.05, -0.1, 1.0), f32))
+    op, bp = (c(n_steps=ev.n_steps[0], stride=stride, lam=lam) for c in (O.Params, B.ScanParams))
+    ref = O.scan(synth.Field(kind=0, b=b), op, seeds, spec.charge, O.wires_aos(wires), ev.hit_offsets, drift, mask, want_dca=True)
+    got = gpu_dca(ctx, B.DeviceField(0, b=b), bp, seeds, spec.charge, wires, ev.hit_offsets, drift, mask, f32, want_dca=False,
+                  use_bounds=use_bounds)
+    e = per_wire_residual(ref["dca"], ev.hit_offsets, drift, mask)
+    assert (np.abs(got["rss"] - ref["rss"]) <= rss_bound(e, lam, FP32_DCA_TOL)).all()
+    assert (np.abs(got["n_in"] - ref["n_in"]) <= (np.abs(e - lam) <= FP32_DCA_TOL).sum(1)).all() and (ref["n_in"] > 0).all()
