@@ -294,11 +294,9 @@ __device__ __forceinline__ void advance_interval(const F &f, const PropArgs &a, 
 // 2^18 seeds and by the issue of one warp per scheduler at a few thousand.  The general loop of
 // propagate_kernel and this, FP32 with spheres: 2^18 seeds x 70 states 101 and 82 us (5.2 TB/s of stores),
 // 2^14 x 2229 386 and 160, 256 x 70 25 and 15; FP64 2^15 x 139 427 and 248.
-// together: the block's warps take a state at a time side by side (see propagate_kernel).
 template <typename T, class F, int STRIDE, typename Off>
 __device__ __forceinline__ void record_inside(const F &f, const PropArgs &a, const AxialStep<T> &ks, T y[6],
-                                              bool valid, int64_t s, int lane, float4 *tab, T R0, T R1,
-                                              bool together)
+                                              bool valid, int64_t s, int lane, float4 *tab, T R0, T R1)
 {
     const int n_rec = a.n_rec, G0 = a.G0, G1 = a.G1;
     const int64_t plane = (int64_t)n_rec * a.S;
@@ -326,13 +324,6 @@ __device__ __forceinline__ void record_inside(const F &f, const PropArgs &a, con
     store();
     int r = 0;
     if (!tab) {
-        if (together) {
-            for (r = 1; r < n_rec; ++r) {
-                __syncthreads();
-                next();
-            }
-            return;
-        }
 #pragma unroll 4
         for (r = 1; r < n_rec; ++r) next();
         return;
@@ -411,16 +402,37 @@ __device__ __forceinline__ void record_inside(const F &f, const PropArgs &a, con
     }
 }
 
+// The same without spheres, the block's warps side by side (TOGETHER, see prop_launch): every warp of the block
+// is here, and n_rec is the launch's, so that each meets as many barriers.
+template <typename T, class F, int STRIDE>
+__device__ __forceinline__ void record_together(const F &f, const PropArgs &a, const AxialStep<T> &ks, T y[6],
+                                                bool valid, int64_t s)
+{
+    const int64_t S = a.S, plane = (int64_t)a.n_rec * S;
+    T *p = (T *)a.points + s;
+    float lo[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    typename F::Cell cell;
+    for (int r = 0; r < a.n_rec; ++r, p += S) {
+        if (r > 0) {
+            __syncthreads();
+            advance_interval<T, F, STRIDE>(f, a, ks, T(0), T(0), T(0), y, lo, cell);
+        }
+        if (valid)
+#pragma unroll
+            for (int c = 0; c < 6; ++c) p[c * plane] = y[c];
+    }
+}
+
 template <class F>
 constexpr bool is_uniform = false;
 template <typename T>
 constexpr bool is_uniform<FieldUniform<T>> = true;
 
 // BATCH: one launch for a batch of events; block b belongs to the event that batch_find gives.
-// Lanes past the last seed repeat it (in a uniform axial field without storing): with idle lanes instead, the shuffles of every
-// sphere found the last warp of a seed count that is no multiple of 32 diverged, and that one warp
+// Lanes past the last seed repeat it (in a uniform axial field without storing): with idle lanes instead, the
+// shuffles of every sphere found the last warp of a seed count that is no multiple of 32 diverged, and that one warp
 // made the launch 4 times as long (10,000 seeds x 140 states: 191 us against 46 us for 9,984).
-template <typename T, class F, int STRIDE, bool BATCH>
+template <typename T, class F, int STRIDE, bool BATCH, bool TOGETHER = false>
 __global__ void __launch_bounds__(128) propagate_kernel(F f, PropArgs a, BatchLaunch L)
 {
     int64_t bx = blockIdx.x;
@@ -482,17 +494,18 @@ __global__ void __launch_bounds__(128) propagate_kernel(F f, PropArgs a, BatchLa
         const AxialStep<float> kf{(float)ks.am1, (float)ks.b, (float)ks.c, (float)ks.d, (float)ks.dz};
         const bool in = stays_inside((float)y[0], (float)y[1], (float)y[2], (float)y[3], (float)y[4], kf, n_rec,
                                      a.lim_f[0], a.lim_f[1], a.lim_f[2], 4e-9f);
-        // Neighbouring warps share 32-byte sectors where a row is no multiple of 32 seeds.  Without spheres
-        // to form, the warps of a block drift apart and those sectors are written in halves; held side by
-        // side by a barrier per state (the block is all inside, so every warp takes this loop): 59,535 FP32
-        // seeds x 275 states 129 -> 98 us, 76,545 x 138 77 -> 56 us.  Whole lines gain nothing.
-        const bool together = !wb && (S & 31) != 0 && blockDim.x > 32 && __syncthreads_and(in);
+        if constexpr (TOGETHER)
+            if (__syncthreads_and(in)) {
+                if (valid) a.n_valid[s] = n_rec;
+                record_together<T, F, STRIDE>(f, a, ks, y, valid, s);
+                return;
+            }
         if (__all_sync(0xffffffffu, in)) {
             if (valid) a.n_valid[s] = n_rec;
             if (plane * (int64_t)sizeof(T) < ((int64_t)1 << 32))
-                record_inside<T, F, STRIDE, uint32_t>(f, a, ks, y, valid, s, lane, tab, R0, R1, together);
+                record_inside<T, F, STRIDE, uint32_t>(f, a, ks, y, valid, s, lane, tab, R0, R1);
             else
-                record_inside<T, F, STRIDE, size_t>(f, a, ks, y, valid, s, lane, tab, R0, R1, together);
+                record_inside<T, F, STRIDE, size_t>(f, a, ks, y, valid, s, lane, tab, R0, R1);
             return;
         }
     }
@@ -756,10 +769,26 @@ cudaError_t launch_lattice_batch(comet_dtype dt, const BatchLaunch &L, cudaStrea
     return cudaGetLastError();
 }
 
+// TOGETHER: neighbouring warps share 32-byte sectors where a row is no multiple of 32 seeds.  Without spheres to
+// form, the warps of a block drift apart and those sectors are written in halves, so blocks whose tracks all stay
+// inside hold their warps side by side by a barrier per state: 59,535 FP32 seeds x 275 states 129 and 97 us,
+// 76,545 x 138 77 and 56.  Whole lines gain nothing.  (A kernel of its own: in the other its code moved the
+// recording of a few seeds by up to 17%.)
 template <typename T, class F, bool BATCH>
 static void prop_launch(const F &fld, const PropArgs &a, int stride, unsigned nb, const BatchLaunch &L,
                         cudaStream_t st, int nt = 128)
 {
+    if constexpr (F::kAxial && !BATCH)
+        if (!a.bounds && (a.S & 31) != 0 && nt > 32) {
+            switch (stride) {
+            case 1: propagate_kernel<T, F, 1, false, true><<<nb, nt, 0, st>>>(fld, a, L); break;
+            case 2: propagate_kernel<T, F, 2, false, true><<<nb, nt, 0, st>>>(fld, a, L); break;
+            case 4: propagate_kernel<T, F, 4, false, true><<<nb, nt, 0, st>>>(fld, a, L); break;
+            case 8: propagate_kernel<T, F, 8, false, true><<<nb, nt, 0, st>>>(fld, a, L); break;
+            default: propagate_kernel<T, F, 0, false, true><<<nb, nt, 0, st>>>(fld, a, L); break;
+            }
+            return;
+        }
     switch (stride) {
     case 1: propagate_kernel<T, F, 1, BATCH><<<nb, nt, 0, st>>>(fld, a, L); break;
     case 2: propagate_kernel<T, F, 2, BATCH><<<nb, nt, 0, st>>>(fld, a, L); break;
