@@ -637,8 +637,8 @@ FP64_PEAK_TFLOPS = 1.25
 # count the recorded states).
 # Valid only for the kernel sources they were measured on (SHA-1 of the package's csrc/ files);
 # reported as null once those change.
-NCU_TRAFFIC = {"csrc_sha1": "4e3dd4393e52b4d843f8a1d7b3ca6aaa9c6a8301", "stride": 32,
-               "dca": 171.5e6, "propagate": 403.7e6}
+NCU_TRAFFIC = {"csrc_sha1": "5bb36bebed4ed30ed43c1ca34c3bc18977a8e919", "stride": 32,
+               "dca": 170.1e6, "propagate": 398.1e6}
 
 
 def csrc_sha1() -> str:

@@ -28,7 +28,8 @@
  *     (row c holds component c of every seed), the seed index running fastest.
  *   - Every call is asynchronous on `stream` (a cudaStream_t; NULL is the legacy default stream) and
  *     returns once its kernels are enqueued.  Arguments are validated on the host before anything is
- *     launched; an invalid argument returns COMET_ERR_INVALID_ARG and launches nothing.  A failed
+ *     launched; an invalid argument returns COMET_ERR_INVALID_ARG and launches nothing (a call of
+ *     several steps, comet_scan_partition, ends at the step that refuses it).  A failed
  *     launch returns COMET_ERR_CUDA.  No call aborts, throws or prints.  comet_last_error() returns
  *     a message for the last non-OK status of the calling thread.
  *   - The library allocates device memory only inside a comet_ctx (comet_scan_select_noalloc
@@ -185,8 +186,8 @@ comet_status comet_scan_lattice(comet_ctx *ctx, comet_dtype dtype, const comet_l
  *            bounds for comet_scan_dca with the same params -- for each group of 32 consecutive
  *            seeds, the bounding spheres (x, y, z, radius) of its track segments (8 super-segments,
  *            24 level-1 segments each; a negative radius marks a segment no seed has, one that is not
- *            a number a segment of a group with a track that is not finite).  Writing them costs a few percent of this call and saves
- *            comet_scan_dca from rebuilding them.
+ *            a number a segment of a group with a track that is not finite).  Writing them costs a
+ *            few percent of this call and saves comet_scan_dca from rebuilding them.
  * One thread extrapolates one seed with fixed-step RK4.  The FP32 path carries each state component
  * as an unevaluated float pair (a compensated sum), so that 6,500 steps stay within a few um of FP64;
  * the recorded value is the leading float.  FP64 in a uniform axial field with fewer than four
